@@ -131,7 +131,7 @@ Workspace plan_workspace(const Shape& s, bool job) {
   L.bvec = take((size_t)L.Ppad * 2 * rs);
   L.A = take((size_t)L.Ppad * L.Ppad * rs);
   L.Linv = take((size_t)L.nT * kNB * kNB * rs);
-  L.sync = take((size_t)chol_sync_ints(L.nT) * 4);
+  L.sync = take((size_t)chol_sync_ints(L.nT, s.prec) * 4);
   L.gains = take(K * N * 8 * rs);
   L.gain_inv = take(N * 8 * rs);
   L.parts = take((size_t)kMaxParts * 8);
@@ -537,7 +537,7 @@ static Workspace plan_lm_block(const Shape& s, int T_max) {
   L.bvec = take((size_t)L.Ppad * 2 * rs);
   L.A = take((size_t)L.Ppad * L.Ppad * rs);
   L.Linv = take((size_t)L.nT * kNB * kNB * rs);
-  L.sync = take((size_t)chol_sync_ints(L.nT) * 4);
+  L.sync = take((size_t)chol_sync_ints(L.nT, s.prec) * 4);
   L.total = o;
   return L;
 }
@@ -854,7 +854,7 @@ static CholWs plan_chol_ws(int n, int prec) {
   L.status = take(256);
   L.A = take((size_t)L.Ppad * L.Ppad * rs);
   L.Linv = take((size_t)L.nT * kNB * kNB * rs);
-  L.sync = take((size_t)chol_sync_ints(L.nT) * 4);
+  L.sync = take((size_t)chol_sync_ints(L.nT, prec) * 4);
   L.bvec = take((size_t)L.Ppad * 2 * rs);
   L.bpad = take((size_t)L.Ppad * 8);
   L.xpad = take((size_t)L.Ppad * 8);
@@ -878,7 +878,7 @@ static int cholesky_impl(int n, R* A, int lda, const double* b, double* x, int k
   SC_CUDA(cudaMemcpy2DAsync(Aw, (size_t)L.Ppad * sizeof(R), A, (size_t)lda * sizeof(R), (size_t)n * sizeof(R), n,
                             cudaMemcpyDeviceToDevice, st));
   SC_CUDA(launch_pad_identity<R>(Aw, L.Ppad, n, st));
-  SC_CUDA(cudaMemsetAsync(sync, 0, (size_t)chol_sync_ints(L.nT) * 4, st));
+  SC_CUDA(cudaMemsetAsync(sync, 0, (size_t)chol_sync_ints(L.nT, sizeof(R) == 4 ? SC_MIXED : SC_FP64) * 4, st));
   prof_start(PK_CHOL, st);
   const cudaError_t ce = launch_chol<R>(Aw, L.Ppad, L.nT, Linv, sync, status, nullptr, 0, kernel, st);
   prof_stop(PK_CHOL, st);

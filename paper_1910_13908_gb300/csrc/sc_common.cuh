@@ -371,11 +371,20 @@ cudaError_t launch_pad_identity(R* A, int Ppad, int n, cudaStream_t st);
 __host__ __device__ int4 chol_task(int nT, int t);   // (type, i, k, j), type -1 past the end
 __host__ __device__ int4 solve_task(int nT, int t);
 int chol_ntasks(int nT);
-int chol_sync_ints(int nT);
+int chol_sync_ints(int nT, int prec);  // size of the sync area
 // kernel: SC_CHOL_SIMT or SC_CHOL_TENSOR (float32 only)
 template <typename R>
 cudaError_t launch_chol(R* A, int lda, int nT, R* Linv, int* sync, uint32_t* status, LMState* lm,
                         int max_ctas, int kernel, cudaStream_t st);
+// chol_f64.cu: the float64 factorisations of the jobs of a batch (G = 1: one
+// matrix), and the solves; nT counts 64x64 tiles
+int chol64_sync_ints(int nT);
+cudaError_t launch_chol64(double* A, int lda, int nT, double* Linv, int* sync, uint32_t* status, LMState* lm,
+                          int max_ctas, cudaStream_t st, const Batch& bt = Batch{});
+cudaError_t launch_solve64(const double* A, int lda, int nT, const double* Linv, int* sync, const double* b,
+                           uint64_t* bwork, double* x, int accumulate, uint32_t tag, uint32_t* status,
+                           const LMState* lm, cudaStream_t st, const Batch& bt = Batch{});
+int chol64_b_task(int n, int j, int idx, int* I, int* K);
 // The factorisations of a whole batch as one persistent launch: the task
 // lists of the G jobs interleaved (task t is task t / G of job t mod G), no
 // walker; every tile is computed by the same arithmetic as in launch_chol.
