@@ -56,9 +56,8 @@ static int ok() {
 
 static size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
 
-// (timeslot, channel) splits of the point-source contraction: enough
-// (station tile pair, split) blocks for two per multiprocessor.
-static int coherency_splits(const Shape& s, int sms) {
+// Ranges of (timeslot, channel) pairs that the float32 sums w_pq are cut into.
+static int w_splits(const Shape& s, int sms) {
   const int nt = (s.N + 63) / 64, tiles = nt * (nt + 1) / 2;
   return std::max(1, std::min(s.T * s.F, (2 * sms + tiles - 1) / tiles));
 }
@@ -89,10 +88,6 @@ Workspace plan_workspace(const Shape& s, bool job) {
   int64_t tb = (int64_t)T * (int64_t)B;
   L.tchunk = (int)std::max<int64_t>(1, std::min<int64_t>((int64_t)T, tb / target));
   L.nchunk = (int)((T + L.tchunk - 1) / L.tchunk);
-  // room for the predict kernel's (timeslot, channel) splits on a GPU of up
-  // to kMaxSMs multiprocessors; the launch takes what the current device
-  // needs (coherency_splits), so the size does not depend on the device
-  L.splits = coherency_splits(s, kMaxSMs);
   size_t o = 0;
   auto take = [&](size_t bytes) {
     size_t at = o;
@@ -103,7 +98,6 @@ Workspace plan_workspace(const Shape& s, bool job) {
   L.lm = take(sizeof(LMState));
   L.C = job ? take(K * T * B * F * 2 * rs) : 0;
   L.w = take((job ? K : 1) * B * rs);
-  L.wpart = take((size_t)L.splits * B * 4);
   L.Rres = job ? take(T * B * F * 8 * rs) : 0;
   L.E = s.prec == SC_MIXED ? take(T * F * Smax * N * 8) : 0;
   L.Sf = take(F * Smax * 8);
@@ -165,7 +159,7 @@ struct Ctx {
   Workspace L;
   char* base;
   cudaStream_t st;
-  int splits;  // coherency splits for the current device (<= L.splits)
+  int splits;  // ranges of the float32 sums w_pq
   template <class T>
   T* at(size_t off) const {
     return reinterpret_cast<T*>(base + off);
@@ -184,7 +178,7 @@ static int open_ctx(Ctx& c, const sc_dims* d, int32_t prec, void* ws, size_t ws_
     return fail(SC_ENOMEM, "workspace of %zu bytes, %zu needed", ws_bytes, c.L.total);
   c.base = static_cast<char*>(ws);
   c.st = static_cast<cudaStream_t>(stream);
-  c.splits = std::min(c.L.splits, coherency_splits(c.s, device_sms()));
+  c.splits = w_splits(c.s, device_sms());
   SC_CUDA(cudaMemsetAsync(c.status(), 0, 256, c.st));
   return SC_OK;
 }
@@ -246,13 +240,12 @@ static int predict_all(const Ctx& c, const double* uvw, const double* freqs, con
     if (s.prec == SC_MIXED) {
       float2* E = c.at<float2>(c.L.E);
       float* Sf = c.at<float>(c.L.Sf);
-      float* wpart = c.at<float>(c.L.wpart);
       SC_LAUNCH(PK_PHASORS, launch_station_phasors(s, uvw, freqs, sky->l + a, sky->m + a, sky->flux + a,
                                      sky->alpha + a, sky->f0, S, E, Sf, c.st));
-      SC_LAUNCH(PK_COHERENCY, launch_coherency_f32(s, S, E, Sf, reinterpret_cast<float2*>(Ck), wpart, c.splits, c.st));
+      SC_LAUNCH(PK_COHERENCY, launch_coherency_f32(s, S, E, Sf, reinterpret_cast<float2*>(Ck), c.st));
       if (w_out)
-        SC_LAUNCH(PK_OTHER, launch_sum_parts(wpart, c.splits, s.B, reinterpret_cast<float*>(w_out) + (size_t)s.B * k,
-                                 c.st));
+        SC_LAUNCH(PK_OTHER, launch_w_splits(s, c.splits, reinterpret_cast<const float2*>(Ck),
+                                            reinterpret_cast<float*>(w_out) + (size_t)s.B * k, c.st));
     } else {
       if (S > 0) {
         SC_LAUNCH(PK_COHERENCY, launch_predict_f64(s, uvw, freqs, sky->l + a, sky->m + a, sky->flux + a, sky->alpha + a,

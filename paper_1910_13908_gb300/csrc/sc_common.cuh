@@ -194,7 +194,6 @@ struct Workspace {
   // job-level buffers
   size_t C;          // [K][T][B][F] complex  (SAGE only)
   size_t w;          // [K][B] real
-  size_t wpart;      // [splits][B] real (predict partial sums)
   size_t Rres;       // [T][B][F][4] complex running residual (SAGE only)
   size_t E;          // [T][F][S_max][N] float2 station phasors (mixed)
   size_t Sf;         // [F][S_max] float fluxes at each channel (mixed)
@@ -223,7 +222,7 @@ struct Workspace {
   size_t srcp;       // [2][F][S_max] float4: spectral Stokes, Gaussian quadratic form
   // consensus across sub-bands (sc_calibrate_consensus)
   size_t pen;        // [K][8N] double, penalty targets of one band's clusters
-  int nT, Ppad, nchunk, tchunk, splits;
+  int nT, Ppad, nchunk, tchunk;
 };
 
 struct Shape {
@@ -295,15 +294,15 @@ cudaError_t launch_station_phasors(const Shape& s, const double* uvw, const doub
                                    const double* l, const double* m, const double* flux,
                                    const double* alpha, double f0, int S, float2* E, float* Sf,
                                    cudaStream_t st);
-cudaError_t launch_coherency_f32(const Shape& s, int S, const float2* E, const float* Sf,
-                                 float2* C, float* wpart, int splits, cudaStream_t st);
+cudaError_t launch_coherency_f32(const Shape& s, int S, const float2* E, const float* Sf, float2* C,
+                                 cudaStream_t st);
+cudaError_t launch_w_splits(const Shape& s, int splits, const float2* C, float* w, cudaStream_t st);
 cudaError_t launch_predict_f64(const Shape& s, const double* uvw, const double* freqs,
                                const double* l, const double* m, const double* flux,
                                const double* alpha, double f0, int S, double2* C,
                                cudaStream_t st);
 template <typename R>
 cudaError_t launch_w_from_C(const Shape& s, const R* C, R* w, cudaStream_t st);
-cudaError_t launch_sum_parts(const float* wpart, int splits, int64_t B, float* w, cudaStream_t st);
 
 // lm_pass.cu
 enum PassFlags { P_OLD = 1, P_SUB = 2, P_WRITE_R = 4, P_STATS = 8 };
