@@ -71,18 +71,22 @@ __global__ void k_source_params(int F, int S, const double* __restrict__ freqs,
 }
 
 constexpr int kFT = 32;  // stations per tile edge
-constexpr int kFS = 32;  // sources staged per step
+constexpr int kFS = 16;  // sources staged per step
 
-__global__ void __launch_bounds__(256) k_coherency_full_f32(int N, int T, int F, int S, int64_t B, int nt,
-                                                             const double* __restrict__ uvw,
-                                                             const float2* __restrict__ E,
-                                                             const float4* __restrict__ st,
-                                                             const float4* __restrict__ gq,
-                                                             float* __restrict__ C) {
-  __shared__ float2 sp_[kFS][kFT];  // e_p,s
-  __shared__ float2 sq_[kFS][kFT];  // e_q,s
-  __shared__ float4 sst[kFS];
-  __shared__ float4 sgq[kFS];
+// Bound by the float32 pipes (twelve FMAs and the shape's exponential per
+// source and baseline) once the staging is out of the way: with 32 sources
+// loaded between two barriers a block waited for global memory at every step
+// (256 stations x 10 timeslots x 1 channel x 50 sources: 83 -> 76 us).
+__global__ void __launch_bounds__(256, 2) k_coherency_full_f32(int N, int T, int F, int S, int64_t B, int nt,
+                                                               const double* __restrict__ uvw,
+                                                               const float2* __restrict__ E,
+                                                               const float4* __restrict__ st,
+                                                               const float4* __restrict__ gq,
+                                                               float* __restrict__ C) {
+  __shared__ float2 sp_[2][kFS][kFT];  // e_p,s
+  __shared__ float2 sq_[2][kFS][kFT];  // e_q,s
+  __shared__ float4 sst[2][kFS];
+  __shared__ float4 sgq[2][kFS];
   int L = blockIdx.x, tp = 0;
   while (L >= nt - tp) {
     L -= nt - tp;
@@ -112,34 +116,53 @@ __global__ void __launch_bounds__(256) k_coherency_full_f32(int N, int T, int F,
 #pragma unroll
     for (int j = 0; j < 2; ++j) aI[i][j] = aQ[i][j] = aU[i][j] = aV[i][j] = make_float2(0.f, 0.f);
 
+  // The next step's phasors and parameters go to registers before this
+  // step's products, and on to shared memory after them.
   const float2* Et = E + (size_t)tf * S * N;
-  for (int s0 = 0; s0 < S; s0 += kFS) {
-    for (int e = threadIdx.x; e < kFS * kFT; e += blockDim.x) {
-      const int ss = e / kFT, c = e % kFT;
-      const int sidx = s0 + ss;
-      float2 va = make_float2(0.f, 0.f), ve = make_float2(0.f, 0.f);
-      if (sidx < S) {
-        if (p0 + c < N) va = Et[(size_t)sidx * N + p0 + c];
-        if (q0 + c < N) ve = Et[(size_t)sidx * N + q0 + c];
-      }
-      sp_[ss][c] = va;
-      sq_[ss][c] = ve;
+  const int c = threadIdx.x % kFT, r0 = threadIdx.x / kFT;  // rows r0, r0 + 8
+  float2 va[2], ve[2];
+  float4 vs, vg;
+  const float2 z2 = make_float2(0.f, 0.f);
+  const float4 z4 = make_float4(0.f, 0.f, 0.f, 0.f);
+  auto fetch = [&](int s0) {
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {
+      const int sidx = s0 + r0 + 8 * u;
+      va[u] = sidx < S && p0 + c < N ? __ldg(Et + (size_t)sidx * N + p0 + c) : z2;
+      ve[u] = sidx < S && q0 + c < N ? __ldg(Et + (size_t)sidx * N + q0 + c) : z2;
     }
     if (threadIdx.x < kFS) {
       const int sidx = s0 + threadIdx.x;
-      sst[threadIdx.x] = sidx < S ? st[(size_t)f * S + sidx] : make_float4(0.f, 0.f, 0.f, 0.f);
-      sgq[threadIdx.x] = sidx < S ? gq[(size_t)f * S + sidx] : make_float4(0.f, 0.f, 0.f, 0.f);
+      vs = sidx < S ? __ldg(st + (size_t)f * S + sidx) : z4;
+      vg = sidx < S ? __ldg(gq + (size_t)f * S + sidx) : z4;
     }
-    __syncthreads();
+  };
+  auto put = [&](int b) {
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {
+      sp_[b][r0 + 8 * u][c] = va[u];
+      sq_[b][r0 + 8 * u][c] = ve[u];
+    }
+    if (threadIdx.x < kFS) {
+      sst[b][threadIdx.x] = vs;
+      sgq[b][threadIdx.x] = vg;
+    }
+  };
+  fetch(0);
+  put(0);
+  int b = 0;
+  for (int s0 = 0; s0 < S; s0 += kFS, b ^= 1) {
+    __syncthreads();  // this step is staged, and the other buffer is free
+    fetch(s0 + kFS);
     const int ns = min(kFS, S - s0);
     for (int ss = 0; ss < ns; ++ss) {
-      const float4 k4 = sst[ss];
-      const float4 g4 = sgq[ss];
+      const float4 k4 = sst[b][ss];
+      const float4 g4 = sgq[b][ss];
       float2 a[2], e[2];
 #pragma unroll
-      for (int i = 0; i < 2; ++i) a[i] = sp_[ss][ty + 16 * i];
+      for (int i = 0; i < 2; ++i) a[i] = sp_[b][ss][ty + 16 * i];
 #pragma unroll
-      for (int j = 0; j < 2; ++j) e[j] = sq_[ss][tx + 16 * j];
+      for (int j = 0; j < 2; ++j) e[j] = sq_[b][ss][tx + 16 * j];
 #pragma unroll
       for (int i = 0; i < 2; ++i)
 #pragma unroll
@@ -164,7 +187,7 @@ __global__ void __launch_bounds__(256) k_coherency_full_f32(int N, int T, int F,
           aV[i][j].y = fmaf(pi, k4.w, aV[i][j].y);
         }
     }
-    __syncthreads();
+    put(b ^ 1);
   }
 #pragma unroll
   for (int i = 0; i < 2; ++i) {
