@@ -76,7 +76,7 @@ constexpr int kFS = 16;  // sources staged per step
 // Bound by the float32 pipes (twelve FMAs and the shape's exponential per
 // source and baseline) once the staging is out of the way: with 32 sources
 // loaded between two barriers a block waited for global memory at every step
-// (256 stations x 10 timeslots x 1 channel x 50 sources: 83 -> 76 us).
+// (256 stations x 10 timeslots x 4 channels x 50 sources: 83 -> 76 us).
 __global__ void __launch_bounds__(256, 2) k_coherency_full_f32(int N, int T, int F, int S, int64_t B, int nt,
                                                                const double* __restrict__ uvw,
                                                                const float2* __restrict__ E,
