@@ -1132,59 +1132,6 @@ __device__ __forceinline__ void tile_async(R* sm, const R* g, int lda) {
 }
 __device__ __forceinline__ void async_commit_empty() { async_commit(); }
 
-// Tile-vector products on a 64x64 tile in shared memory (pitch 64 + 16
-// bytes), laid out so that each quarter-warp's 16-byte loads hit all 32
-// banks once.
-//
-// mv_rows: out[r] = sum_m T[r][m] v[m].  The quad of lanes 4r..4r+3 owns
-// row r; lane `part` reads the row's 16-byte chunks part + 4u, rotated by
-// three chunks on odd rows (odd rows start 4 banks further on, so the two
-// rows of a quarter-warp then cover distinct banks).  Two shuffles combine
-// the quad; every lane of it returns the row total.
-__device__ __forceinline__ float mv_rows(const float* Tm, const float* v) {
-  constexpr int LD = Pitch<float>::value;
-  const int r = threadIdx.x >> 2, part = threadIdx.x & 3, rot = 3 * (r & 1);
-  float s = 0.f;
-#pragma unroll
-  for (int u = 0; u < 4; ++u) {
-    const int ch = (part + 4 * u + rot) & 15;
-    const float4 t = *reinterpret_cast<const float4*>(Tm + r * LD + 4 * ch);
-    const float4 w = *reinterpret_cast<const float4*>(v + 4 * ch);
-    s = fmaf(t.x, w.x, fmaf(t.y, w.y, fmaf(t.z, w.z, fmaf(t.w, w.w, s))));
-  }
-  s += __shfl_xor_sync(0xffffffffu, s, 1);
-  s += __shfl_xor_sync(0xffffffffu, s, 2);
-  return s;
-}
-
-// mv_cols: out[c] = sum_m T[m][c] v[m] for the columns c = 4g..4g+3 of lane
-// group g = tid / 16.  Lane mr of the group takes rows m = mr + 16k: a
-// quarter-warp reads eight consecutive rows (4 banks apart) at one column
-// offset.  Four butterfly rounds combine the group; every lane of it
-// returns the four totals.
-template <typename R>
-__device__ __forceinline__ void mv_cols(const R* Tm, const R* v, R (&o)[4]) {
-  constexpr int LD = Pitch<R>::value;
-  const int g = threadIdx.x >> 4, mr = threadIdx.x & 15;
-  R a0 = 0, a1 = 0, a2 = 0, a3 = 0;
-#pragma unroll
-  for (int k = 0; k < 4; ++k) {
-    const int m = mr + 16 * k;
-    const R* t = Tm + m * LD + 4 * g;
-    const R w = v[m];
-    const float4 q = *reinterpret_cast<const float4*>(t);
-    a0 = fma((R)q.x, w, a0), a1 = fma((R)q.y, w, a1), a2 = fma((R)q.z, w, a2), a3 = fma((R)q.w, w, a3);
-  }
-#pragma unroll
-  for (int d = 1; d < 16; d <<= 1) {
-    a0 += __shfl_xor_sync(0xffffffffu, a0, d);
-    a1 += __shfl_xor_sync(0xffffffffu, a1, d);
-    a2 += __shfl_xor_sync(0xffffffffu, a2, d);
-    a3 += __shfl_xor_sync(0xffffffffu, a3, d);
-  }
-  o[0] = a0, o[1] = a1, o[2] = a2, o[3] = a3;
-}
-
 // C = A B for 64x64 tiles in shared memory (all with the tile pitch), 256
 // threads with 4x4 outputs each: A is read as a broadcast per half-warp, B
 // along contiguous rows.
@@ -1418,6 +1365,8 @@ cudaError_t launch_chol_solve(const R* A, int lda, int nT, const R* Linv, int* s
   if constexpr (sizeof(R) == 8) {
     return launch_solve64(A, lda, nT, Linv, sync, b, bwork, x, accumulate, 2 * e, status, lm, st, bt);
   } else {
+    if (const int nc = solve_cluster_size(nT, bt.G))
+      return launch_chol_solve_cluster(A, lda, nT, nc, Linv, b, x, accumulate, status, lm, st, bt);
     int n_tasks = 2 * nT;
     if ((long long)n_tasks * bt.G > (1LL << 30)) return cudaErrorInvalidValue;
     size_t smem = sizeof(R) * (4 * kNB * Pitch<R>::value + kNB);

@@ -384,6 +384,12 @@ cudaError_t launch_solve64(const double* A, int lda, int nT, const double* Linv,
                            uint64_t* bwork, double* x, int accumulate, uint32_t tag, uint32_t* status,
                            const LMState* lm, cudaStream_t st, const Batch& bt = Batch{});
 int chol64_b_task(int n, int j, int idx, int* I, int* K);
+// CTAs of the cluster that solves one of G float32 systems of nT tile rows
+// (0: k_chol_solve takes the call), and that solve.
+int solve_cluster_size(int nT, int G);
+cudaError_t launch_chol_solve_cluster(const float* A, int lda, int nT, int nc, const float* Linv, const double* b,
+                                      double* x, int accumulate, uint32_t* status, const LMState* lm, cudaStream_t st,
+                                      const Batch& bt);
 // The factorisations of a whole batch as one persistent launch: the task
 // lists of the G jobs interleaved (task t is task t / G of job t mod G), no
 // walker; every tile is computed by the same arithmetic as in launch_chol.
