@@ -178,6 +178,14 @@ __global__ void __launch_bounds__(256, SlabOf<R>::MINB) k_residual_all(int N, in
 // so a warp's 8-byte reads are conflict-free.  Requires K >= S: the
 // visibility slot of an item is refilled only after its first stage has
 // been consumed.
+//
+// What bounds it is the issue of instructions at 16 warps per SM (HBM runs at
+// 0.7 of its rate), so they are what is saved: an item is five timeslots of a
+// (baseline, channel) pair, whose loads are contiguous across a warp and need
+// no addresses of their own, and the products run on pairs of floats (three
+// instructions per entry instead of six).  512 stations x 10 timeslots x 4
+// channels, 40 clusters: 545 us with items of four channels, 443 with
+// timeslots, 405 with pairs.
 
 namespace {
 __device__ __forceinline__ void ra_cp8(void* dst, const void* src) {
@@ -193,72 +201,132 @@ template <int W>
 __device__ __forceinline__ void ra_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(W) : "memory"); }
 }  // namespace
 
-constexpr int kPipeNV = 4;     // visibilities per item
 constexpr int kPipeThreads = 256;
+constexpr int kPipeStages = 4;
+constexpr int kPipeMaxNV = 5;  // timeslots per item at most
 
-template <int S>
+template <int NV>
 constexpr size_t pipe_smem_bytes() {
-  return (size_t)S * kPipeNV * kPipeThreads * 8 + (size_t)kPipeNV * 2 * kPipeThreads * 16;
+  return (size_t)kPipeStages * NV * kPipeThreads * 8 + (size_t)NV * 2 * kPipeThreads * 16;
 }
 
-template <typename IX, int S>
+// Pairs of float32 in one register pair; each half rounds like the scalar
+// instruction.
+namespace {
+using f32x2 = unsigned long long;
+__device__ __forceinline__ f32x2 pack2(float lo, float hi) {
+  f32x2 r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+  return r;
+}
+__device__ __forceinline__ float2 unpack2(f32x2 v) {
+  float2 r;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
+  return r;
+}
+__device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b) {
+  f32x2 r;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b) {
+  f32x2 r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
+  f32x2 r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
+}  // namespace
+
+// An item: nt x nf = NV timeslots x channels of a baseline, in nslab slabs of
+// the timeslots and ngrp groups of the channels.
+struct PipeSplit {
+  int nt, nf, nslab, ngrp;
+};
+
+template <typename IX, int NV>
 __global__ void __launch_bounds__(kPipeThreads, 2) k_residual_all_pipe(
-    int N, int T, int F, int64_t B, int K, int nslab, const float* V, const float* __restrict__ C,
+    int N, int T, int F, int64_t B, int K, PipeSplit sp, const float* V, const float* __restrict__ C,
     const float* __restrict__ Jr, const float* __restrict__ Jinv, float* Rout,
     double* __restrict__ part) {
-  constexpr int NV = kPipeNV;
+  constexpr int S = kPipeStages;
   extern __shared__ __align__(16) unsigned char ra_smem[];
   float2* ring = reinterpret_cast<float2*>(ra_smem);                                  // [S][NV][T]
   float4* vslot = reinterpret_cast<float4*>(ra_smem + (size_t)S * NV * kPipeThreads * 8);  // [2NV][T]
   const int tid = threadIdx.x;
-  const int TF = T * F;
-  const int64_t n_items = (int64_t)nslab * B;
-  const int64_t stride = (int64_t)gridDim.x * kPipeThreads;
-  const IX per_cluster = (IX)TF * (IX)B;
-
-  // visibility offsets (t*B + b)*F + f of item idx's NV (t, f) pairs
-  auto offsets = [&](int64_t idx, IX* off, int& nv) {
-    const int slab = (int)(idx / B);
-    const int64_t b = idx - (int64_t)slab * B;
-    const int r0 = slab * NV;
-    nv = min(NV, TF - r0);
-    int t = r0 / F, f = r0 - t * F;
+  const IX BF = (IX)B * (IX)F;  // elements of one timeslot
+  // five elements are five timeslots: constants here leave the registers
+  constexpr bool kTimes = NV == kPipeMaxNV;
+  const IX cols = kTimes ? BF : (IX)B * (IX)sp.ngrp, n_items = (IX)sp.nslab * cols;
+  const IX stride = (IX)gridDim.x * kPipeThreads;
+  const size_t per_cluster = (size_t)T * (size_t)BF;
+  const int nf = kTimes ? 1 : sp.nf, nt = kTimes ? NV : sp.nt;
+  IX steps[NV];  // from an item's first element to its others
 #pragma unroll
-    for (int i = 0; i < NV; ++i) {
-      off[i] = ((IX)t * (IX)B + (IX)b) * (IX)F + (IX)f;
-      if (++f == F) {
-        f = 0;
-        ++t;
-      }
+  for (int i = 0; i < NV; ++i) steps[i] = (IX)(i / nf) * BF + (IX)(i % nf);
+  auto step = [&](int i) -> size_t { return kTimes ? (size_t)((IX)i * BF) : (size_t)steps[i]; };
+
+  // item idx: its baseline, its first element and which of its elements exist
+  auto has = [](unsigned live, int i) { return kTimes ? i < (int)live : (bool)(live >> i & 1); };
+  auto locate = [&](IX idx, IX& b, IX& off, unsigned& live) {
+    const IX slab = idx / cols, col = idx - slab * cols;
+    const int t0 = (int)slab * nt;
+    if (kTimes) {
+      b = col / (IX)F;
+      off = (IX)t0 * BF + col;
+      live = min(NV, T - t0);
+      return;
+    }
+    b = col / (IX)sp.ngrp;
+    const int f0 = (int)(col - b * (IX)sp.ngrp) * nf;
+    off = (IX)t0 * BF + b * (IX)F + (IX)f0;
+    live = (1u << NV) - 1;
+    if (t0 + nt > T || f0 + nf > F) {
+      live = 0;
+      for (int i = 0; i < NV; ++i)
+        if (t0 + i / nf < T && f0 + i % nf < F) live |= 1u << i;
     }
   };
 
   // prefetch cursor: (pf_idx, pf_k), S steps ahead of the arithmetic
-  int64_t pf_idx = (int64_t)blockIdx.x * kPipeThreads + tid;
-  int pf_k = 0, pf_nv = 0, pf_stage = 0;
-  IX pf_off[NV];
-  if (pf_idx < n_items) offsets(pf_idx, pf_off, pf_nv);
-  auto issue = [&]() {
+  IX pf_idx = (IX)blockIdx.x * kPipeThreads + tid;
+  int pf_k = 0, pf_stage = 0;
+  unsigned pf_live = 0;
+  IX pf_off = 0;
+  const float* pf_c = C;
+  auto seek = [&]() {
+    pf_live = 0;
     if (pf_idx < n_items) {
-      const float* Ck = C + (IX)2 * (IX)pf_k * per_cluster;
+      IX b;
+      locate(pf_idx, b, pf_off, pf_live);
+      pf_c = C + 2 * (size_t)pf_off;
+    }
+  };
+  seek();
+  auto issue = [&]() {
+    float2* dst = ring + pf_stage * NV * kPipeThreads + tid;
+#pragma unroll
+    for (int i = 0; i < NV; ++i)
+      if (has(pf_live, i)) ra_cp8(dst + i * kPipeThreads, pf_c + 2 * step(i));
+    if (pf_k == 0) {
+      const float* Vi = V + 8 * (size_t)pf_off;
 #pragma unroll
       for (int i = 0; i < NV; ++i)
-        if (i < pf_nv) ra_cp8(&ring[((size_t)pf_stage * NV + i) * kPipeThreads + tid], Ck + 2 * pf_off[i]);
-      if (pf_k == 0) {
-#pragma unroll
-        for (int i = 0; i < NV; ++i)
-          if (i < pf_nv) {
-            ra_cp16(&vslot[(2 * i) * kPipeThreads + tid], V + 8 * pf_off[i]);
-            ra_cp16(&vslot[(2 * i + 1) * kPipeThreads + tid], V + 8 * pf_off[i] + 4);
-          }
-      }
+        if (has(pf_live, i)) {
+          ra_cp16(&vslot[(2 * i) * kPipeThreads + tid], Vi + 8 * step(i));
+          ra_cp16(&vslot[(2 * i + 1) * kPipeThreads + tid], Vi + 8 * step(i) + 4);
+        }
     }
     ra_commit();
     pf_stage = pf_stage + 1 == S ? 0 : pf_stage + 1;
+    pf_c += 2 * per_cluster;
     if (++pf_k == K) {
       pf_k = 0;
       pf_idx += stride;
-      if (pf_idx < n_items) offsets(pf_idx, pf_off, pf_nv);
+      seek();
     }
   };
 #pragma unroll 1
@@ -267,49 +335,63 @@ __global__ void __launch_bounds__(kPipeThreads, 2) k_residual_all_pipe(
   double cost = 0.0;
   int stage = 0;
 #pragma unroll 1
-  for (int64_t idx = (int64_t)blockIdx.x * kPipeThreads + tid; idx < n_items; idx += stride) {
-    IX off[NV];
-    int nv;
-    offsets(idx, off, nv);
-    const int64_t b = idx % B;
+  for (IX idx = (IX)blockIdx.x * kPipeThreads + tid; idx < n_items; idx += stride) {
+    IX off, b;
+    unsigned live;
+    locate(idx, b, off, live);
     int p, q;
-    bl_pair(b, N, p, q);
-    m22<float> acc[NV];
-    m22<float> Jp = ld_vis(Jr + 8 * (size_t)p), Jq = ld_vis(Jr + 8 * (size_t)q);
+    bl_pair((int64_t)b, N, p, q);
+    f32x2 acc[NV][4];
+    unsigned jp = p, jq = q;  // rows of Jr
+    m22<float> Jp = ld_vis(Jr + 8 * (size_t)jp), Jq = ld_vis(Jr + 8 * (size_t)jq);
 #pragma unroll 1
     for (int k = 0; k < K; ++k) {
       const m22<float> G = mul_h(Jp, Jq);
+      // c G = (cr gr - ci gi, cr gi + ci gr) as cr (gr, gi) + ci (-gi, gr)
+      const f32x2 g[4] = {pack2(G.a.re, G.a.im), pack2(G.b.re, G.b.im), pack2(G.c.re, G.c.im), pack2(G.d.re, G.d.im)};
+      const f32x2 h[4] = {pack2(-G.a.im, G.a.re), pack2(-G.b.im, G.b.re), pack2(-G.c.im, G.c.re),
+                          pack2(-G.d.im, G.d.re)};
       if (k + 1 < K) {
-        Jp = ld_vis(Jr + 8 * ((size_t)(k + 1) * N + p));
-        Jq = ld_vis(Jr + 8 * ((size_t)(k + 1) * N + q));
+        jp += N;
+        jq += N;
+        Jp = ld_vis(Jr + 8 * (size_t)jp);
+        Jq = ld_vis(Jr + 8 * (size_t)jq);
       }
       ra_wait<S - 1>();
       if (k == 0) {
 #pragma unroll
         for (int i = 0; i < NV; ++i) {
           const float4 u = vslot[(2 * i) * kPipeThreads + tid], w = vslot[(2 * i + 1) * kPipeThreads + tid];
-          acc[i] = {{u.x, u.y}, {u.z, u.w}, {w.x, w.y}, {w.z, w.w}};
+          acc[i][0] = pack2(u.x, u.y), acc[i][1] = pack2(u.z, u.w);
+          acc[i][2] = pack2(w.x, w.y), acc[i][3] = pack2(w.z, w.w);
         }
       }
+      const float2* src = ring + stage * NV * kPipeThreads + tid;
 #pragma unroll
       for (int i = 0; i < NV; ++i) {
-        const float2 c = ring[((size_t)stage * NV + i) * kPipeThreads + tid];
-        acc[i] = acc[i] - smul(cx<float>{c.x, c.y}, G);
+        const float2 c = src[i * kPipeThreads];
+        const f32x2 nr = pack2(-c.x, -c.x), ni = pack2(-c.y, -c.y);
+#pragma unroll
+        for (int e = 0; e < 4; ++e) acc[i][e] = add2(acc[i][e], fma2(nr, g[e], mul2(ni, h[e])));
       }
       stage = stage + 1 == S ? 0 : stage + 1;
       issue();
     }
+    m22<float> r[NV];
 #pragma unroll
-    for (int i = 0; i < NV; ++i)
-      if (i < nv) cost += (double)frob2(acc[i]);
+    for (int i = 0; i < NV; ++i) {
+      const float2 e0 = unpack2(acc[i][0]), e1 = unpack2(acc[i][1]), e2 = unpack2(acc[i][2]), e3 = unpack2(acc[i][3]);
+      r[i] = {{e0.x, e0.y}, {e1.x, e1.y}, {e2.x, e2.y}, {e3.x, e3.y}};
+      if (has(live, i)) cost += (double)frob2(r[i]);
+    }
     if (Jinv != nullptr) {
       const m22<float> Ip = ld_vis(Jinv + 8 * (size_t)p), Iq = ld_vis(Jinv + 8 * (size_t)q);
 #pragma unroll
-      for (int i = 0; i < NV; ++i) acc[i] = mul_h(mul(Ip, acc[i]), Iq);
+      for (int i = 0; i < NV; ++i) r[i] = mul_h(mul(Ip, r[i]), Iq);
     }
 #pragma unroll
     for (int i = 0; i < NV; ++i)
-      if (i < nv) st_vis(Rout + 8 * off[i], acc[i]);
+      if (has(live, i)) st_vis(Rout + 8 * ((size_t)off + step(i)), r[i]);
   }
   ra_wait<0>();
   if (part == nullptr) return;
@@ -333,8 +415,6 @@ cudaError_t launch_gain_prep(const Shape& s, const double* J, int corr, R* Jr, R
   return cudaGetLastError();
 }
 
-constexpr int kPipeStages = 4;
-
 // resident blocks of a kernel at the given block size and dynamic shared memory
 template <typename Kern>
 static int resident_blocks(Kern kern, int threads, size_t smem) {
@@ -345,25 +425,57 @@ static int resident_blocks(Kern kern, int threads, size_t smem) {
   return std::max(1, sms * std::max(per, 1));
 }
 
-template <typename IX>
-static cudaError_t go_pipe(const Shape& s, const float* V, const float* C, const float* Jr,
-                          const float* Jinv, float* Rout, double* part, int max_parts, int* n_parts,
-                          cudaStream_t st) {
-  constexpr int S = kPipeStages;
-  constexpr size_t smem = pipe_smem_bytes<S>();
+template <typename IX, int NV>
+static cudaError_t go_pipe(const Shape& s, const PipeSplit& sp, const float* V, const float* C, const float* Jr,
+                           const float* Jinv, float* Rout, double* part, int max_parts, int* n_parts,
+                           cudaStream_t st) {
+  constexpr size_t smem = pipe_smem_bytes<NV>();
+  const auto kern = k_residual_all_pipe<IX, NV>;
   // per device and cheap: set on every launch
-  cudaError_t e = cudaFuncSetAttribute(k_residual_all_pipe<IX, S>,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  static const int resident = resident_blocks(k_residual_all_pipe<IX, S>, kPipeThreads, smem);
-  const int nslab = (s.T * s.F + kPipeNV - 1) / kPipeNV;
-  const int64_t n_items = (int64_t)nslab * s.B;
+  static const int resident = resident_blocks(kern, kPipeThreads, smem);
+  const int64_t n_items = (int64_t)sp.nslab * sp.ngrp * s.B;
   const int grid = (int)std::min<int64_t>(
       std::min<int64_t>((n_items + kPipeThreads - 1) / kPipeThreads, resident), max_parts);
-  k_residual_all_pipe<IX, S><<<grid, kPipeThreads, smem, st>>>(s.N, s.T, s.F, s.B, s.K, nslab, V, C, Jr,
-                                                               Jinv, Rout, part);
+  kern<<<grid, kPipeThreads, smem, st>>>(s.N, s.T, s.F, s.B, s.K, sp, V, C, Jr, Jinv, Rout, part);
   *n_parts = grid;
   return cudaGetLastError();
+}
+
+// The split with the most visibilities per item, since an item forms its
+// baseline's G once per cluster: five timeslots, or up to four as timeslots x
+// channels.  Timeslots alone, whose loads are contiguous across a warp, unless
+// channels give a tenth more (2 x 2 of 2 timeslots x 4 channels: 73 us, 2 x 1:
+// 99, at 512 stations and 20 clusters); items of three count less (6 x 4 in
+// items of 2 x 2: 167 us, of 3 x 1: 220).
+static PipeSplit pipe_split(int T, int F) {
+  auto even = [](int n, int cap, int& parts) { parts = (n + cap - 1) / cap; return (n + parts - 1) / parts; };
+  PipeSplit best{};
+  double most = 0.0;
+  for (int c = 0; c <= std::min(F, kPipeMaxNV - 1); ++c) {
+    PipeSplit p;
+    p.nf = even(F, std::max(c, 1), p.ngrp);
+    p.nt = even(T, c == 0 ? kPipeMaxNV : (kPipeMaxNV - 1) / p.nf, p.nslab);
+    const double vis = (double)T * F / ((double)p.nslab * p.ngrp) * (p.nf > 1 ? 0.9 : 1.0) *
+                       (p.nt * p.nf == 3 ? 0.85 : 1.0);
+    if (vis > most) most = vis, best = p;
+  }
+  return best;
+}
+
+template <typename IX>
+static cudaError_t pick_pipe(const Shape& s, const float* V, const float* C, const float* Jr,
+                             const float* Jinv, float* Rout, double* part, int max_parts, int* n_parts,
+                             cudaStream_t st) {
+  const PipeSplit sp = pipe_split(s.T, s.F);
+  switch (sp.nt * sp.nf) {
+    case 1: return go_pipe<IX, 1>(s, sp, V, C, Jr, Jinv, Rout, part, max_parts, n_parts, st);
+    case 2: return go_pipe<IX, 2>(s, sp, V, C, Jr, Jinv, Rout, part, max_parts, n_parts, st);
+    case 3: return go_pipe<IX, 3>(s, sp, V, C, Jr, Jinv, Rout, part, max_parts, n_parts, st);
+    case 4: return go_pipe<IX, 4>(s, sp, V, C, Jr, Jinv, Rout, part, max_parts, n_parts, st);
+    default: return go_pipe<IX, 5>(s, sp, V, C, Jr, Jinv, Rout, part, max_parts, n_parts, st);
+  }
 }
 
 template <typename R>
@@ -375,8 +487,8 @@ cudaError_t launch_residual_all(const Shape& s, const R* V, const R* C, const R*
   if constexpr (sizeof(R) == 4) {
     if (s.K >= kPipeStages) {
       return top_ < (1ull << 31)
-                 ? go_pipe<uint32_t>(s, V, C, Jr, Jinv, Rout, part, max_parts, n_parts, st)
-                 : go_pipe<size_t>(s, V, C, Jr, Jinv, Rout, part, max_parts, n_parts, st);
+                 ? pick_pipe<uint32_t>(s, V, C, Jr, Jinv, Rout, part, max_parts, n_parts, st)
+                 : pick_pipe<size_t>(s, V, C, Jr, Jinv, Rout, part, max_parts, n_parts, st);
     }
   }
   static const int resident = [] {
