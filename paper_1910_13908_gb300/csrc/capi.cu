@@ -327,6 +327,7 @@ static int lm_solve(const Ctx& c, const R* Xin, bool running, const R* C, const 
   R* Linv = c.at<R>(L.Linv);
   uint64_t* bw = c.at<uint64_t>(L.bvec);
   int* sync = c.at<int>(L.sync);
+  const int n_sync = chol_sync_ints(L.nT, s.prec);
   LMState* lm = c.lm();
 
   SC_CUDA(cudaMemcpyAsync(J_old, J_io, n8, cudaMemcpyDeviceToDevice, c.st));
@@ -341,8 +342,9 @@ static int lm_solve(const Ctx& c, const R* Xin, bool running, const R* C, const 
                                           c.st));
   SC_LAUNCH(PK_LM, launch_lm_init(lm, &o, s.N, b, b.J_cur, c.st));
   for (int it = 0; it < o.n_lm; ++it) {
-    SC_LAUNCH(PK_ASSEMBLE, launch_assemble<R>(s, L.Ppad, L.Ppad, w, Jr, b.H_cur, lm, A, true, false, c.st));
-    SC_LAUNCH(PK_CHOL, launch_chol<R>(A, L.Ppad, L.nT, Linv, sync, c.status(), lm, o.max_ctas, o.chol_kernel, c.st));
+    SC_LAUNCH(PK_ASSEMBLE, launch_assemble<R>(s, L.Ppad, L.Ppad, w, Jr, b.H_cur, lm, A, true, false, c.st, Batch{}, sync,
+                                              n_sync));
+    SC_LAUNCH(PK_CHOL, launch_chol<R>(A, L.Ppad, L.nT, Linv, sync, c.status(), lm, o.max_ctas, o.chol_kernel, c.st, true));
     SC_LAUNCH(PK_SOLVE, launch_chol_solve<R>(A, L.Ppad, L.nT, Linv, sync, b.g_cur, bw, x, 0, c.status(), lm, c.st));
     if (mixed) {
       for (int sw = 0; sw < o.refine_sweeps; ++sw) {
@@ -598,6 +600,7 @@ static int sage_batched(const Ctx& c, const std::vector<Ctx>& jc, const sc_job* 
   R* Linv = c.at<R>(L.Linv);
   uint64_t* bw = c.at<uint64_t>(L.bvec);
   int* sync = c.at<int>(L.sync);
+  const int n_sync = chol_sync_ints(L.nT, s.prec);
   LMState* lm = c.lm();
   const int* nchunk_dev = &lm->nchunk;
   auto blk = [&](int g) { return c.base + (size_t)g * js; };
@@ -644,9 +647,10 @@ static int sage_batched(const Ctx& c, const std::vector<Ctx>& jc, const sc_job* 
                                               nullptr, 0.0, c.st, bt));
       SC_LAUNCH(PK_LM, launch_lm_init(lm, &o.lm, s.N, b, b.J_cur, c.st, bt));
       for (int it = 0; it < o.lm.n_lm; ++it) {
-        SC_LAUNCH(PK_ASSEMBLE, launch_assemble<R>(s, L.Ppad, L.Ppad, w, Jr, b.H_cur, lm, A, true, false, c.st, bt));
+        SC_LAUNCH(PK_ASSEMBLE, launch_assemble<R>(s, L.Ppad, L.Ppad, w, Jr, b.H_cur, lm, A, true, false, c.st, bt, sync,
+                                                  n_sync));
         SC_LAUNCH(PK_CHOL, launch_chol_batch<R>(A, L.Ppad, L.nT, Linv, sync, c.status(), lm, o.lm.max_ctas, bt,
-                                                order, c.st));
+                                                order, c.st, true));
         SC_LAUNCH(PK_SOLVE, launch_chol_solve<R>(A, L.Ppad, L.nT, Linv, sync, b.g_cur, bw, x, 0, c.status(), lm,
                                                  c.st, bt));
         if (mixed) {

@@ -568,6 +568,7 @@ __global__ void __launch_bounds__(kThr) k_solve64(const double* __restrict__ A0,
                                                  const double* __restrict__ b0, uint64_t* __restrict__ yw0,
                                                  double* __restrict__ x0, int accumulate, uint32_t tag_fwd,
                                                  uint32_t* status0, const LMState* lm0, int G, size_t js) {
+  dep_sync(js == 0);
   const uint32_t tag_bwd = tag_fwd + 1;
   __shared__ __align__(16) double D[kSB * kSLD], B[2][kSB * kSLD];
   __shared__ double vin[kSB];
@@ -695,7 +696,7 @@ __global__ void __launch_bounds__(kThr) k_solve64(const double* __restrict__ A0,
 }  // namespace
 
 cudaError_t launch_chol64(double* A, int lda, int nT, double* Linv, int* sync, uint32_t* status, LMState* lm,
-                          int max_ctas, cudaStream_t st, const Batch& bt) {
+                          int max_ctas, cudaStream_t st, bool zeroed, const Batch& bt) {
   // up to four blocks per SM: the float64 pipes take about one, the others
   // cover claims, waits and loads (one block of four groups per SM with
   // blocks kept for P was 4% slower at order 1200 and 15% at 4096)
@@ -708,7 +709,9 @@ cudaError_t launch_chol64(double* A, int lda, int nT, double* Linv, int* sync, u
   }();
   const int n = tiles64(nT);
   const size_t row = sizeof(int) * chol64_sync_ints(nT);
-  cudaError_t e = bt.G == 1 ? cudaMemsetAsync(sync, 0, row, st) : cudaMemset2DAsync(sync, bt.js, 0, row, bt.G, st);
+  cudaError_t e = zeroed      ? cudaSuccess
+                  : bt.G == 1 ? cudaMemsetAsync(sync, 0, row, st)
+                              : cudaMemset2DAsync(sync, bt.js, 0, row, bt.G, st);
   if (e != cudaSuccess) return e;
   // per job: the walker and as many blocks as the first panel has tasks, at
   // least one, within what is resident at once
@@ -716,6 +719,8 @@ cudaError_t launch_chol64(double* A, int lda, int nT, double* Linv, int* sync, u
   const int total = max_ctas > 0 ? std::min(resident, max_ctas) : resident;
   const int per_job = (int)std::max<long long>(2, std::min<long long>(1 + tasks, total / bt.G));
   if ((long long)per_job * bt.G > (1LL << 30)) return cudaErrorInvalidValue;
+  // not by launch_dep: blocks that come in while the assembly still runs crowd
+  // on the SMs it has left, the walker among them (64 stations: 4.58 ms, 3.81)
   k_chol64<<<per_job * bt.G, kBlock64, 0, st>>>(A, lda, n, Linv, per_job, bt.js, sync, status, lm);
   return cudaGetLastError();
 }
@@ -727,9 +732,8 @@ cudaError_t launch_solve64(const double* A, int lda, int nT, const double* Linv,
   if ((long long)2 * nS * bt.G > (1LL << 30)) return cudaErrorInvalidValue;
   const cudaError_t e = cudaMemsetAsync(sync + 1, 0, sizeof(int), st);
   if (e != cudaSuccess) return e;
-  k_solve64<<<2 * nS * bt.G, kThr, 0, st>>>(A, lda, nS, Linv, sync, b, bwork, x, accumulate, tag, status, lm, bt.G,
-                                           bt.js);
-  return cudaGetLastError();
+  return launch_dep(bt.js == 0, k_solve64, 2 * nS * bt.G, kThr, 0, st, A, lda, nS, Linv, sync, b, bwork, x, accumulate, tag, status,
+                    lm, bt.G, bt.js);
 }
 
 // Host view of the enumeration: B task idx of panel j of n tiles as (I, K);

@@ -201,6 +201,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_chol_solve_cluster(const float*
                                                                     const double* __restrict__ b,
                                                                     double* __restrict__ x, int accumulate,
                                                                     uint32_t* status, const LMState* lm, size_t js) {
+  dep_sync(js == 0);
   const int NC = gridDim.x, c = blockIdx.x, job = blockIdx.y;  // one cluster per job
   lm = job_ptr(lm, js, job);
   if (lm != nullptr && (lm->done | lm->notpd)) return;  // the whole cluster alike
@@ -439,12 +440,14 @@ cudaError_t launch_chol_solve_cluster(const float* A, int lda, int nT, int nc, c
   cfg.blockDim = dim3(kThreads, 1, 1);
   cfg.dynamicSmemBytes = kSmem;
   cfg.stream = st;
-  cudaLaunchAttribute at[1];
+  cudaLaunchAttribute at[2];
   at[0].id = cudaLaunchAttributeClusterDimension;
   at[0].val.clusterDim.x = nc;
   at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+  at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;  // as launch_dep
+  at[1].val.programmaticStreamSerializationAllowed = bt.js == 0;
   cfg.attrs = at;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = 2;
   return cudaLaunchKernelEx(&cfg, k_chol_solve_cluster, A, lda, nT, Linv, b, x, accumulate, status, lm, bt.js);
 }
 

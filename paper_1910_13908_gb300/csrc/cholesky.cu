@@ -350,6 +350,7 @@ template <typename R>
 __global__ void __launch_bounds__(kCholThreads) k_chol(R* __restrict__ A, int lda, int nT,
                                                       R* __restrict__ Linv, int n_tasks,
                                                       int* sync, uint32_t* status, LMState* lm) {
+  dep_sync(true);
   if (lm != nullptr && lm->done) return;
   constexpr int LD = Pitch<R>::value;
   extern __shared__ __align__(16) unsigned char smraw[];
@@ -710,6 +711,7 @@ __global__ void __launch_bounds__(kCholThreads, 2) k_chol_tc(const __grid_consta
                                                         const __grid_constant__ CUtensorMap tmL, float* __restrict__ A,
                                                         int lda, int nT, float* __restrict__ Linv, int n_tasks,
                                                         int* sync, uint32_t* status, LMState* lm) {
+  dep_sync(true);
   if (lm != nullptr && lm->done) return;
   extern __shared__ unsigned char smraw[];
   // 1024-byte alignment of the operand region, whatever precedes the dynamic array
@@ -1000,7 +1002,7 @@ static int chol_tc_grid() {
 }
 
 static cudaError_t launch_chol_tc(float* A, int lda, int nT, float* Linv, int* sync, uint32_t* status, LMState* lm,
-                                  int max_ctas, cudaStream_t st) {
+                                  int max_ctas, cudaStream_t st, bool zeroed) {
   const int n_tasks = chol_ntasks(nT);
   CUtensorMap tmA, tmL;
   cudaError_t e = encode_tile_map(&tmA, A, (uint64_t)lda, (uint64_t)nT * kNB, (uint64_t)lda * sizeof(float));
@@ -1009,34 +1011,33 @@ static cudaError_t launch_chol_tc(float* A, int lda, int nT, float* Linv, int* s
   if (e != cudaSuccess) return e;
   int grid = std::min(chol_tc_grid(), n_tasks);
   if (max_ctas > 0) grid = std::min(grid, max_ctas);
-  e = cudaMemsetAsync(sync, 0, sizeof(int) * chol_factor_reset_ints(nT), st);
+  if (!zeroed) e = cudaMemsetAsync(sync, 0, sizeof(int) * chol_factor_reset_ints(nT), st);
   if (e != cudaSuccess) return e;
-  k_chol_tc<<<grid, kCholThreads, chol_tc_smem(), st>>>(tmA, tmL, A, lda, nT, Linv, n_tasks, sync, status, lm);
-  return cudaGetLastError();
+  return launch_dep(true, k_chol_tc, grid, kCholThreads, chol_tc_smem(), st, tmA, tmL, A, lda, nT, Linv, n_tasks, sync, status,
+                    lm);
 }
 
 template <typename R>
 cudaError_t launch_chol(R* A, int lda, int nT, R* Linv, int* sync, uint32_t* status, LMState* lm,
-                        int max_ctas, int kernel, cudaStream_t st) {
+                        int max_ctas, int kernel, cudaStream_t st, bool zeroed) {
   if constexpr (sizeof(R) == 8) {
-    return launch_chol64(A, lda, nT, Linv, sync, status, lm, max_ctas, st);
+    return launch_chol64(A, lda, nT, Linv, sync, status, lm, max_ctas, st, zeroed);
   } else {
-    if (kernel == SC_CHOL_TENSOR) return launch_chol_tc(A, lda, nT, Linv, sync, status, lm, max_ctas, st);
+    if (kernel == SC_CHOL_TENSOR) return launch_chol_tc(A, lda, nT, Linv, sync, status, lm, max_ctas, st, zeroed);
     int n_tasks = chol_ntasks(nT);
     size_t smem = sizeof(R) * (4 * kNB) * Pitch<R>::value;  // two buffer pairs; the walker uses 3.5 tiles
     const void* fn = reinterpret_cast<const void*>(&k_chol<R>);
     int grid = std::min(chol_grid<R>(fn, smem), n_tasks);
     if (max_ctas > 0) grid = std::min(grid, max_ctas);
-    cudaError_t e = cudaMemsetAsync(sync, 0, sizeof(int) * chol_factor_reset_ints(nT), st);
+    cudaError_t e = zeroed ? cudaSuccess : cudaMemsetAsync(sync, 0, sizeof(int) * chol_factor_reset_ints(nT), st);
     if (e != cudaSuccess) return e;
-    k_chol<R><<<grid, kCholThreads, smem, st>>>(A, lda, nT, Linv, n_tasks, sync, status, lm);
-    return cudaGetLastError();
+    return launch_dep(true, k_chol<R>, grid, kCholThreads, smem, st, A, lda, nT, Linv, n_tasks, sync, status, lm);
   }
 }
 template cudaError_t launch_chol<float>(float*, int, int, float*, int*, uint32_t*, LMState*, int, int,
-                                        cudaStream_t);
+                                        cudaStream_t, bool);
 template cudaError_t launch_chol<double>(double*, int, int, double*, int*, uint32_t*, LMState*, int, int,
-                                         cudaStream_t);
+                                         cudaStream_t, bool);
 
 // Blocks of k_chol_batch: as many as are resident at once, computed once.
 template <typename R>
@@ -1057,12 +1058,12 @@ static int chol_batch_grid(size_t smem) {
 
 template <typename R>
 cudaError_t launch_chol_batch(R* A, int lda, int nT, R* Linv, int* sync, uint32_t* status, LMState* lm,
-                              int max_ctas, const Batch& bt, const uint32_t* order, cudaStream_t st) {
+                              int max_ctas, const Batch& bt, const uint32_t* order, cudaStream_t st, bool zeroed) {
   if constexpr (sizeof(R) == 8) {
     // the task order is that of the float32 kernel's combined list; here
     // every job has blocks of its own
     if (bt.G < 1) return cudaErrorInvalidValue;
-    return launch_chol64(A, lda, nT, Linv, sync, status, lm, max_ctas, st, bt);
+    return launch_chol64(A, lda, nT, Linv, sync, status, lm, max_ctas, st, zeroed, bt);
   } else {
     const int n_tasks = chol_ntasks(nT);
     if (bt.G < 1 || (long long)n_tasks * bt.G > (1LL << 30)) return cudaErrorInvalidValue;
@@ -1072,7 +1073,9 @@ cudaError_t launch_chol_batch(R* A, int lda, int nT, R* Linv, int* sync, uint32_
     if (max_ctas > 0) grid = std::min(grid, max_ctas);
     // every job's counters: rows of the reset length at the job stride
     const size_t row = sizeof(int) * chol_factor_reset_ints(nT);
-    cudaError_t e = bt.G == 1 ? cudaMemsetAsync(sync, 0, row, st) : cudaMemset2DAsync(sync, bt.js, 0, row, bt.G, st);
+    cudaError_t e = zeroed      ? cudaSuccess
+                    : bt.G == 1 ? cudaMemsetAsync(sync, 0, row, st)
+                                : cudaMemset2DAsync(sync, bt.js, 0, row, bt.G, st);
     if (e != cudaSuccess) return e;
     k_chol_batch<R><<<grid, kCholThreads, smem, st>>>(A, lda, nT, Linv, n_tasks, bt.G, bt.js, order, sync, status,
                                                        lm);
@@ -1080,9 +1083,9 @@ cudaError_t launch_chol_batch(R* A, int lda, int nT, R* Linv, int* sync, uint32_
   }
 }
 template cudaError_t launch_chol_batch<float>(float*, int, int, float*, int*, uint32_t*, LMState*, int,
-                                              const Batch&, const uint32_t*, cudaStream_t);
+                                              const Batch&, const uint32_t*, cudaStream_t, bool);
 template cudaError_t launch_chol_batch<double>(double*, int, int, double*, int*, uint32_t*, LMState*, int,
-                                               const Batch&, const uint32_t*, cudaStream_t);
+                                               const Batch&, const uint32_t*, cudaStream_t, bool);
 
 // The combined task list of a batch's factorisations, the jobs staggered
 // over a window of W jobs.  Job g's task t (of n per job) gets the key
@@ -1213,6 +1216,7 @@ __global__ void __launch_bounds__(kCholThreads) k_chol_solve(const R* __restrict
                                                             int accumulate, uint32_t tag_fwd,
                                                             uint32_t* status0, const LMState* lm0, int G,
                                                             size_t js) {
+  dep_sync(js == 0);
   constexpr int LD = Pitch<R>::value;
   const uint32_t tag_bwd = tag_fwd + 1;
   extern __shared__ __align__(16) unsigned char smraw[];
@@ -1379,9 +1383,8 @@ cudaError_t launch_chol_solve(const R* A, int lda, int nT, const R* Linv, int* s
     SyncView sv(sync, nT);
     cudaError_t err = cudaMemsetAsync(sv.sctr, 0, sizeof(int), st);
     if (err != cudaSuccess) return err;
-    k_chol_solve<R><<<n_tasks * bt.G, kCholThreads, smem, st>>>(A, lda, nT, Linv, n_tasks, sync, b, bwork, x,
-                                                                accumulate, 2 * e, status, lm, bt.G, bt.js);
-    return cudaGetLastError();
+    return launch_dep(bt.js == 0, k_chol_solve<R>, n_tasks * bt.G, kCholThreads, smem, st, A, lda, nT, Linv, n_tasks, sync, b, bwork, x,
+                      accumulate, 2 * e, status, lm, bt.G, bt.js);
   }
 }
 template cudaError_t launch_chol_solve<float>(const float*, int, int, const float*, int*,

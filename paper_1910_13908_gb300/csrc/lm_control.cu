@@ -52,6 +52,7 @@ __device__ __forceinline__ unsigned long long abs_bits(double x) {
 }
 
 __global__ void k_lm_init(LMState* lm, sc_lm_opts o, int N, LMBufs b, const double* __restrict__ J_src, size_t js) {
+  dep_sync(js == 0);
   const int job = blockIdx.z;
   lm = job_ptr(lm, js, job);
   b = job_bufs(b, js, job);
@@ -93,14 +94,14 @@ __global__ void k_lm_init(LMState* lm, sc_lm_opts o, int N, LMBufs b, const doub
 
 cudaError_t launch_lm_init(LMState* lm, const sc_lm_opts* o, int N, const LMBufs& b, const double* J_src,
                            cudaStream_t st, const Batch& bt) {
-  k_lm_init<<<dim3(1, 1, bt.G), 512, 0, st>>>(lm, *o, N, b, J_src, bt.js);
-  return cudaGetLastError();
+  return launch_dep(bt.js == 0, k_lm_init, dim3(1, 1, bt.G), 512, 0, st, lm, *o, N, b, J_src, bt.js);
 }
 
 // One thread per parameter: theta_trial = theta + d, and per block the
 // partial predicted decrease sum d (mu d + g).
 __global__ void __launch_bounds__(kTrialThreads) k_lm_trial(LMState* lm, int N, const double* __restrict__ x,
                                                           LMBufs b, size_t js) {
+  dep_sync(js == 0);
   const int job = blockIdx.z;
   lm = job_ptr(lm, js, job);
   if (lm->done) return;
@@ -132,11 +133,11 @@ int lm_trial_blocks(int N) { return (8 * N + kTrialThreads - 1) / kTrialThreads;
 
 cudaError_t launch_lm_trial(LMState* lm, int N, const double* x, const LMBufs& b, cudaStream_t st,
                             const Batch& bt) {
-  k_lm_trial<<<dim3(lm_trial_blocks(N), 1, bt.G), kTrialThreads, 0, st>>>(lm, N, x, b, bt.js);
-  return cudaGetLastError();
+  return launch_dep(bt.js == 0, k_lm_trial, dim3(lm_trial_blocks(N), 1, bt.G), kTrialThreads, 0, st, lm, N, x, b, bt.js);
 }
 
 __global__ void k_lm_decide(LMState* lm, int N, int n_pred, LMBufs b, size_t js) {
+  dep_sync(js == 0);
   const int job = blockIdx.z;
   lm = job_ptr(lm, js, job);
   if (lm->done) return;
@@ -195,13 +196,13 @@ __global__ void k_lm_decide(LMState* lm, int N, int n_pred, LMBufs b, size_t js)
 }
 
 cudaError_t launch_lm_decide(LMState* lm, int N, const LMBufs& b, cudaStream_t st, const Batch& bt) {
-  k_lm_decide<<<dim3(1, 1, bt.G), 512, 0, st>>>(lm, N, lm_trial_blocks(N), b, bt.js);
-  return cudaGetLastError();
+  return launch_dep(bt.js == 0, k_lm_decide, dim3(1, 1, bt.G), 512, 0, st, lm, N, lm_trial_blocks(N), b, bt.js);
 }
 
 __global__ void k_lm_finish(const LMState* __restrict__ lm, const double* __restrict__ J_cur, int N,
                             double* __restrict__ J_out, double* __restrict__ cost_out,
                             int32_t* __restrict__ iters_out) {
+  dep_sync(true);
   for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < 8 * N; k += gridDim.x * blockDim.x)
     J_out[k] = J_cur[k];
   if (blockIdx.x == 0 && threadIdx.x == 0) {
@@ -212,8 +213,7 @@ __global__ void k_lm_finish(const LMState* __restrict__ lm, const double* __rest
 
 cudaError_t launch_lm_finish(const LMState* lm, const double* J_cur, int N, double* J_out,
                              double* cost_out, int32_t* iters_out, cudaStream_t st) {
-  k_lm_finish<<<(8 * N + 255) / 256, 256, 0, st>>>(lm, J_cur, N, J_out, cost_out, iters_out);
-  return cudaGetLastError();
+  return launch_dep(true, k_lm_finish, (8 * N + 255) / 256, 256, 0, st, lm, J_cur, N, J_out, cost_out, iters_out);
 }
 
 }  // namespace sc

@@ -538,6 +538,7 @@ __global__ void __launch_bounds__(kST * kST) k_lm_eval(int N, int64_t B, int nS,
                                                      const double* __restrict__ J, double* __restrict__ part,
                                                      const LMState* __restrict__ lm, size_t js,
                                                      const int* __restrict__ nchunk_dev) {
+  dep_sync(js == 0);
   const int job = blockIdx.z;
   lm = job_ptr(lm, js, job);
   if (lm != nullptr && (lm->done | lm->skip)) return;
@@ -614,9 +615,8 @@ cudaError_t launch_lm_eval(const Shape& s, bool sub, const double* stat, int nch
                            const LMState* lm, cudaStream_t st, const Batch& bt, const int* nchunk_dev) {
   const int nS = (s.N + kST - 1) / kST, pairs = nS * (nS + 1) / 2;
   const dim3 grd(pairs, 1, bt.G);
-  if (sub) k_lm_eval<R, true><<<grd, kST * kST, 0, st>>>(s.N, s.B, nS, nchunk, stat, J, part, lm, bt.js, nchunk_dev);
-  else k_lm_eval<R, false><<<grd, kST * kST, 0, st>>>(s.N, s.B, nS, nchunk, stat, J, part, lm, bt.js, nchunk_dev);
-  return cudaGetLastError();
+  return launch_dep(bt.js == 0, sub ? k_lm_eval<R, true> : k_lm_eval<R, false>, grd, kST * kST, 0, st, s.N, s.B, nS, nchunk, stat, J,
+                    part, lm, bt.js, nchunk_dev);
 }
 template cudaError_t launch_lm_eval<float>(const Shape&, bool, const double*, int, const double*, double*,
                                            const LMState*, cudaStream_t, const Batch&, const int*);
@@ -640,6 +640,7 @@ __global__ void __launch_bounds__(kSumThreads) k_station_sum(int N, int nS, cons
                                                              const LMState* __restrict__ lm,
                                                              const double* __restrict__ pen, double pen_w,
                                                              size_t js) {
+  dep_sync(js == 0);
   const int job = blockIdx.z;
   lm = job_ptr(lm, js, job);
   if (lm != nullptr && (lm->done | lm->skip)) return;
@@ -706,8 +707,7 @@ cudaError_t launch_station_sum(const Shape& s, const double* part, const double*
   const int nS = (s.N + kST - 1) / kST;
   const unsigned blocks = (unsigned)((s.N + kSumThreads / 32 - 1) / (kSumThreads / 32));
   const dim3 grd(blocks, 1, bt.G);
-  k_station_sum<<<grd, kSumThreads, 0, st>>>(s.N, nS, part, J, g, H, cpart, gmax, lm, pen, pen_w, bt.js);
-  return cudaGetLastError();
+  return launch_dep(bt.js == 0, k_station_sum, grd, kSumThreads, 0, st, s.N, nS, part, J, g, H, cpart, gmax, lm, pen, pen_w, bt.js);
 }
 
 }  // namespace sc

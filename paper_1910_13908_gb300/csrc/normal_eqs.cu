@@ -41,9 +41,13 @@ __global__ void __launch_bounds__(256) k_assemble(int N, int lda, int Ppad, cons
                                                   const R* __restrict__ J,
                                                   const double* __restrict__ H,
                                                   const LMState* __restrict__ lm, R* __restrict__ A,
-                                                  int damp, int full, size_t js) {
+                                                  int damp, int full, size_t js, int* zero, int n_zero, bool early) {
+  dep_sync(early);
   const int job = blockIdx.z;
   lm = job_ptr(lm, js, job);
+  if (zero != nullptr && blockIdx.x == 0)
+    for (int i = blockIdx.y * blockDim.x + threadIdx.x; i < n_zero; i += gridDim.y * blockDim.x)
+      job_ptr(zero, js, job)[i] = 0;
   if (lm != nullptr && lm->done) return;
   w = job_ptr(w, js, job);
   J = job_ptr(J, js, job);
@@ -125,18 +129,20 @@ cudaError_t launch_round_jones(const double* J, float* Jf, int n, cudaStream_t s
 template <typename R>
 cudaError_t launch_assemble(const Shape& s, int lda, int Ppad, const R* w, const R* J,
                             const double* H, const LMState* lm, R* A, bool damp, bool full,
-                            cudaStream_t st, const Batch& bt) {
+                            cudaStream_t st, const Batch& bt, int* zero, int n_zero) {
   int groups = (Ppad + 3) / 4;
   dim3 grd((groups + 127) / 128, Ppad, bt.G);
-  k_assemble<R><<<grd, 128, 0, st>>>(s.N, lda, Ppad, w, J, H, lm, A, damp ? 1 : 0, full ? 1 : 0, bt.js);
-  return cudaGetLastError();
+  // up to one wave of blocks: launch_dep
+  const bool early = bt.js == 0 && (long long)grd.x * grd.y <= 16 * 152;
+  return launch_dep(early, k_assemble<R>, grd, 128, 0, st, s.N, lda, Ppad, w, J, H, lm, A, damp ? 1 : 0, full ? 1 : 0,
+                    bt.js, zero, n_zero, early);
 }
 template cudaError_t launch_assemble<float>(const Shape&, int, int, const float*, const float*,
                                             const double*, const LMState*, float*, bool, bool,
-                                            cudaStream_t, const Batch&);
+                                            cudaStream_t, const Batch&, int*, int);
 template cudaError_t launch_assemble<double>(const Shape&, int, int, const double*, const double*,
                                              const double*, const LMState*, double*, bool, bool,
-                                             cudaStream_t, const Batch&);
+                                             cudaStream_t, const Batch&, int*, int);
 
 // Ones on the diagonal of rows n..Ppad-1 of a zeroed padded matrix, so that
 // the padding factorises as the identity.
@@ -172,6 +178,7 @@ __global__ void __launch_bounds__(256) k_refine_prep(int N, const double* __rest
                                                      const double* __restrict__ x,
                                                      const LMState* __restrict__ lm, double* __restrict__ Y,
                                                      size_t js) {
+  dep_sync(js == 0);
   const int job = blockIdx.z;
   lm = job_ptr(lm, js, job);
   if (lm->done | lm->notpd) return;
@@ -196,6 +203,7 @@ __global__ void __launch_bounds__(32 * kRefineWarps) k_refine_residual(int N, co
                                                          const double* __restrict__ Y,
                                                          const LMState* __restrict__ lm,
                                                          double* __restrict__ r, size_t js) {
+  dep_sync(js == 0);
   const int job = blockIdx.z;
   lm = job_ptr(lm, js, job);
   if (lm->done | lm->notpd) return;
@@ -251,11 +259,10 @@ template <typename R>
 cudaError_t launch_refine_residual(const Shape& s, const R* w, const double* J, const double* H,
                                    const double* g, const double* x, const LMState* lm,
                                    double* Y, double* r, cudaStream_t st, const Batch& bt) {
-  k_refine_prep<<<dim3((s.N + 255) / 256, 1, bt.G), 256, 0, st>>>(s.N, J, x, lm, Y, bt.js);
-  cudaError_t e = cudaGetLastError();
+  cudaError_t e = launch_dep(bt.js == 0, k_refine_prep, dim3((s.N + 255) / 256, 1, bt.G), 256, 0, st, s.N, J, x, lm, Y, bt.js);
   if (e != cudaSuccess) return e;
-  k_refine_residual<R><<<dim3(s.N, 1, bt.G), 32 * kRefineWarps, 0, st>>>(s.N, w, J, H, g, x, Y, lm, r, bt.js);
-  return cudaGetLastError();
+  return launch_dep(bt.js == 0, k_refine_residual<R>, dim3(s.N, 1, bt.G), 32 * kRefineWarps, 0, st, s.N, w, J, H, g, x, Y, lm, r,
+                    bt.js);
 }
 template cudaError_t launch_refine_residual<float>(const Shape&, const float*, const double*,
                                                    const double*, const double*, const double*,

@@ -141,6 +141,38 @@ __device__ __forceinline__ void bl_pair(int64_t b, int N, int& p, int& q) {
   q = (int)(b - row_start(pp, N)) + pp + 1;
 }
 
+// ---- launches that overlap the end of the kernel before them ----------------------
+//
+// An LM iteration is about a dozen small kernels, each needing the one before
+// it.  launch_dep(early) lets a kernel's blocks take their places while the
+// previous kernel of the stream runs (programmatic dependent launch), and
+// dep_sync, the first statement of every kernel launched that way, waits until
+// that kernel has completed and its stores are visible; only then may the
+// blocks of the kernel after this one come in, so at most one kernel waits in
+// place.  An iteration of 64 stations takes 192 us instead of 215, of 128 323
+// instead of 345.  A batch's launches and large assemblies, whose many short
+// blocks the two instructions would slow down (batch of 64 jobs: 1.6%), go the
+// plain way: early is given to the kernel and to its launch alike.
+__device__ __forceinline__ void dep_sync(bool early) {
+  if (!early) return;
+  cudaGridDependencySynchronize();
+  cudaTriggerProgrammaticLaunchCompletion();
+}
+template <typename... P, typename... A>
+cudaError_t launch_dep(bool early, void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A... a) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = early ? 1 : 0;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(a)...);
+}
+
 // ---- device LM state ---------------------------------------------------------------
 
 struct LMState {
@@ -350,11 +382,12 @@ cudaError_t launch_residual_all(const Shape& s, const R* V, const R* C, const R*
                                 cudaStream_t st);
 
 // normal_eqs.cu
-// J: the Jones in the matrix's type (rounded once in float32)
+// J: the Jones in the matrix's type (rounded once in float32); zero: n_zero
+// counters to clear with it (the factorisation's, whatever lm says)
 template <typename R>
 cudaError_t launch_assemble(const Shape& s, int lda, int Ppad, const R* w, const R* J,
                             const double* H, const LMState* lm, R* A, bool damp, bool full,
-                            cudaStream_t st, const Batch& bt = Batch{});
+                            cudaStream_t st, const Batch& bt = Batch{}, int* zero = nullptr, int n_zero = 0);
 cudaError_t launch_round_jones(const double* J, float* Jf, int n, cudaStream_t st);
 // r = g - (J^T J + mu I) x in float64; Y [8N] is scratch
 template <typename R>
@@ -371,15 +404,16 @@ __host__ __device__ int4 chol_task(int nT, int t);   // (type, i, k, j), type -1
 __host__ __device__ int4 solve_task(int nT, int t);
 int chol_ntasks(int nT);
 int chol_sync_ints(int nT, int prec);  // size of the sync area
-// kernel: SC_CHOL_SIMT or SC_CHOL_TENSOR (float32 only)
+// kernel: SC_CHOL_SIMT or SC_CHOL_TENSOR (float32 only); zeroed: the kernel
+// before has cleared all of sync
 template <typename R>
 cudaError_t launch_chol(R* A, int lda, int nT, R* Linv, int* sync, uint32_t* status, LMState* lm,
-                        int max_ctas, int kernel, cudaStream_t st);
+                        int max_ctas, int kernel, cudaStream_t st, bool zeroed = false);
 // chol_f64.cu: the float64 factorisations of the jobs of a batch (G = 1: one
 // matrix), and the solves; nT counts 64x64 tiles
 int chol64_sync_ints(int nT);
 cudaError_t launch_chol64(double* A, int lda, int nT, double* Linv, int* sync, uint32_t* status, LMState* lm,
-                          int max_ctas, cudaStream_t st, const Batch& bt = Batch{});
+                          int max_ctas, cudaStream_t st, bool zeroed, const Batch& bt = Batch{});
 cudaError_t launch_solve64(const double* A, int lda, int nT, const double* Linv, int* sync, const double* b,
                            uint64_t* bwork, double* x, int accumulate, uint32_t tag, uint32_t* status,
                            const LMState* lm, cudaStream_t st, const Batch& bt = Batch{});
@@ -395,7 +429,8 @@ cudaError_t launch_chol_solve_cluster(const float* A, int lda, int nT, int nc, c
 // walker; every tile is computed by the same arithmetic as in launch_chol.
 template <typename R>
 cudaError_t launch_chol_batch(R* A, int lda, int nT, R* Linv, int* sync, uint32_t* status, LMState* lm,
-                              int max_ctas, const Batch& bt, const uint32_t* order, cudaStream_t st);
+                              int max_ctas, const Batch& bt, const uint32_t* order, cudaStream_t st,
+                              bool zeroed = false);
 // The combined task order of a batch with the jobs staggered over a window
 // of W jobs: entry m is job << 20 | task (order [G * chol_ntasks(nT)]).
 // Possible when batch_order_ok (G <= 4096, at most 2^20 tasks per job);
