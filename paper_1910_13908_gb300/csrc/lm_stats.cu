@@ -463,6 +463,7 @@ __device__ __forceinline__ void eval_baseline(const double* stat, int64_t B, int
   FF v[kStatV];
 #pragma unroll
   for (int i = 0; i < kStatV; ++i) v[i] = {0.f, 0.f};
+#pragma unroll 4  // the loads of four chunks in flight
   for (int c = 0; c < nchunk; ++c) {
     const float* src = st + (size_t)c * 2 * kStatV * B + b;
 #pragma unroll
