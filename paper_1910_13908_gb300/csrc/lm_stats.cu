@@ -456,9 +456,10 @@ size_t lm_part_doubles(int N) {
 // chunks).  float32 statistics: pair arithmetic with G = J_p J_q^H formed in
 // float32 (the model the visibility pass would form), so the three terms of
 // the cost are those of one and the same G; rho is returned rounded.
+struct NoBuf {};
 __device__ __forceinline__ void eval_baseline(const double* stat, int64_t B, int nchunk, int64_t b, bool sub,
                                               const m22<float>& Jp, const m22<float>& Jq, FF& cost,
-                                              m22<float>& rho, float& W) {
+                                              m22<float>& rho, float& W, NoBuf&) {
   const float* st = reinterpret_cast<const float*>(stat);
   FF v[kStatV];
 #pragma unroll
@@ -490,9 +491,70 @@ __device__ __forceinline__ void eval_baseline(const double* stat, int64_t B, int
   cost = ff_add(ff_add(v[0], ff_mul_f(cross, -2.f)), ff_mul(v[9], g2));
   rho = {{r[0], r[1]}, {r[2], r[3]}, {r[4], r[5]}, {r[6], r[7]}};
 }
+// The same for launches of up to two blocks per SM.  They run the code once, so
+// its length is their time (every line comes from L2): the chunks and the eight
+// entries of G are loops, the latter with the thread's numbers in shared memory,
+// and the next chunk's loads go out before the current one is added.  An LM
+// iteration of 64 stations (10 blocks, 10 chunks) 184 -> 175 us; a batch of 16
+// jobs of 256 (2176 blocks) is 0.4% faster the other way, at three blocks more
+// per SM.
+struct EvalBuf {
+  float2 v[kStatV][kST * kST];  // rhoX and W, pairs
+  float g[8][kST * kST];        // G, then rho
+};
+__device__ __forceinline__ void eval_baseline(const double* stat, int64_t B, int nchunk, int64_t b, bool sub,
+                                              const m22<float>& Jp, const m22<float>& Jq, FF& cost,
+                                              m22<float>& rho, float& W, EvalBuf& eb) {
+  const float* src = reinterpret_cast<const float*>(stat) + b;
+  FF v[kStatV], nx[kStatV];
+#pragma unroll
+  for (int i = 0; i < kStatV; ++i) v[i] = {0.f, 0.f}, nx[i] = {0.f, 0.f};
+  auto load = [&]() {
+#pragma unroll
+    for (int i = 0; i < kStatV; ++i) nx[i] = {src[(size_t)(2 * i) * B], src[(size_t)(2 * i + 1) * B]};
+    src += (size_t)2 * kStatV * B;
+  };
+  if (nchunk > 0) load();
+#pragma unroll 1
+  for (int c = 0; c < nchunk; ++c) {
+    FF cur[kStatV];
+#pragma unroll
+    for (int i = 0; i < kStatV; ++i) cur[i] = nx[i];
+    if (c + 1 < nchunk) load();
+#pragma unroll
+    for (int i = 0; i < kStatV; ++i) v[i] = ff_add(v[i], cur[i]);
+  }
+  W = v[9].hi;
+  if (!sub) {
+    cost = v[0];
+    rho = {{v[1].hi, v[2].hi}, {v[3].hi, v[4].hi}, {v[5].hi, v[6].hi}, {v[7].hi, v[8].hi}};
+    return;
+  }
+  const int tid = threadIdx.x;
+  const m22<float> G = mul_h(Jp, Jq);
+  eb.g[0][tid] = G.a.re, eb.g[1][tid] = G.a.im, eb.g[2][tid] = G.b.re, eb.g[3][tid] = G.b.im;
+  eb.g[4][tid] = G.c.re, eb.g[5][tid] = G.c.im, eb.g[6][tid] = G.d.re, eb.g[7][tid] = G.d.im;
+#pragma unroll
+  for (int i = 1; i < 9; ++i) eb.v[i][tid] = make_float2(v[i].hi, v[i].lo);
+  // cost = S - 2 Re <G, rhoX> + W |G|^2,  rho = rhoX - W G
+  FF cross = {0.f, 0.f}, g2 = {0.f, 0.f};
+#pragma unroll 1
+  for (int k = 0; k < 8; ++k) {
+    const float2 x = eb.v[1 + k][tid];
+    const FF vk = {x.x, x.y};
+    const float g = eb.g[k][tid];
+    cross = ff_add(cross, ff_mul_f(vk, g));
+    g2 = ff_add(g2, two_prod(g, g));
+    const FF rk = ff_add(vk, ff_mul_f(v[9], -g));
+    eb.g[k][tid] = __fadd_rn(rk.hi, rk.lo);
+  }
+  cost = ff_add(ff_add(v[0], ff_mul_f(cross, -2.f)), ff_mul(v[9], g2));
+  rho = {{eb.g[0][tid], eb.g[1][tid]}, {eb.g[2][tid], eb.g[3][tid]}, {eb.g[4][tid], eb.g[5][tid]},
+         {eb.g[6][tid], eb.g[7][tid]}};
+}
 __device__ __forceinline__ void eval_baseline(const double* stat, int64_t B, int nchunk, int64_t b, bool sub,
                                               const m22<double>& Jp, const m22<double>& Jq, double& cost,
-                                              m22<double>& rho, double& W) {
+                                              m22<double>& rho, double& W, NoBuf&) {
   double v[kStatV];
 #pragma unroll
   for (int i = 0; i < kStatV; ++i) v[i] = 0.0;
@@ -533,7 +595,7 @@ template <typename R> struct CostT;
 template <> struct CostT<float> { using T = FF; __device__ static FF zero() { return {0.f, 0.f}; } };
 template <> struct CostT<double> { using T = double; __device__ static double zero() { return 0.0; } };
 
-template <typename R, bool SUB>
+template <typename R, bool SUB, typename Buf>
 __global__ void __launch_bounds__(kST * kST) k_lm_eval(int N, int64_t B, int nS, int nchunk,
                                                      const double* __restrict__ stat,
                                                      const double* __restrict__ J, double* __restrict__ part,
@@ -548,6 +610,7 @@ __global__ void __launch_bounds__(kST * kST) k_lm_eval(int N, int64_t B, int nS,
   part = job_ptr(part, js, job);
   if (nchunk_dev != nullptr) nchunk = *job_ptr(nchunk_dev, js, job);
   __shared__ R colbuf[kColV][kST][kST + 1];
+  __shared__ Buf eb;
   const int pair = blockIdx.x;
   // tile pairs (Pt, Qt), Pt <= Qt, are numbered like the baselines of nS + 1
   // stations: pair = bl_index(Pt, Qt + 1, nS + 1)
@@ -563,7 +626,7 @@ __global__ void __launch_bounds__(kST * kST) k_lm_eval(int N, int64_t B, int nS,
   if (act) {
     Jp = load_jones<R>(J, p);
     Jq = load_jones<R>(J, q);
-    eval_baseline(stat, B, nchunk, bl_index(p, q, N), SUB, Jp, Jq, cost, rh, w);
+    eval_baseline(stat, B, nchunk, bl_index(p, q, N), SUB, Jp, Jq, cost, rh, w, eb);
   }
   double* out = part + (size_t)pair * kPartStride;
   // station p's part, summed over the tile row: the kST lanes of a half-warp
@@ -616,8 +679,10 @@ cudaError_t launch_lm_eval(const Shape& s, bool sub, const double* stat, int nch
                            const LMState* lm, cudaStream_t st, const Batch& bt, const int* nchunk_dev) {
   const int nS = (s.N + kST - 1) / kST, pairs = nS * (nS + 1) / 2;
   const dim3 grd(pairs, 1, bt.G);
-  return launch_dep(bt.js == 0, sub ? k_lm_eval<R, true> : k_lm_eval<R, false>, grd, kST * kST, 0, st, s.N, s.B, nS, nchunk, stat, J,
-                    part, lm, bt.js, nchunk_dev);
+  auto kern = sub ? k_lm_eval<R, true, NoBuf> : k_lm_eval<R, false, NoBuf>;
+  if constexpr (sizeof(R) == 4)
+    if (sub && (long long)pairs * bt.G <= 2 * 152) kern = k_lm_eval<R, true, EvalBuf>;
+  return launch_dep(bt.js == 0, kern, grd, kST * kST, 0, st, s.N, s.B, nS, nchunk, stat, J, part, lm, bt.js, nchunk_dev);
 }
 template cudaError_t launch_lm_eval<float>(const Shape&, bool, const double*, int, const double*, double*,
                                            const LMState*, cudaStream_t, const Batch&, const int*);
