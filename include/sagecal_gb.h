@@ -190,7 +190,7 @@ SC_API int32_t sc_workspace_size(const sc_dims* d, int32_t prec, size_t* bytes);
 SC_API int32_t sc_device_status(const void* ws, size_t ws_bytes, uint32_t* status);
 
 /* Diagnostic, host only (launches nothing): the task order of the tiled
- * Cholesky factorisation (which = 0) or of the two triangular solves
+ * float32 Cholesky factorisation (which = 0) or of the two triangular solves
  * (which = 1) on an nT x nT grid of 64x64 tiles, as (type, i, k, j)
  * quadruples written to out[0 .. 4*cap).  Types: 0 POTRF(j), 1 TRSM(i, j),
  * 2 UPDATE(i, k, j), 3 forward solve of tile row i, 4 backward solve of tile
@@ -569,7 +569,8 @@ SC_API int32_t sc_batched_workspace_size(const sc_dims* dims, int32_t n_jobs, in
  * waiting on one job's dependency chain are few among those working on the
  * others).  window W in [1, 2^20] staggers the jobs instead: job g starts
  * its list when job g - W is about to finish, so that about W matrices are
- * read at a time; sc_tune_batched measures the choices.  ws:
+ * read at a time; sc_tune_batched measures the choices.  In SC_FP64 every
+ * job's factorisation has blocks of its own and the window has no effect.  ws:
  * sc_batched_workspace_size bytes, 256-byte aligned, device memory owned by
  * the caller.  Everything runs on `stream`, after what is already queued on
  * each job's stream, and each job's stream then waits for the batch
