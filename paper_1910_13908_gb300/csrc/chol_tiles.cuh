@@ -1,4 +1,4 @@
-// Pieces shared by the factorisation and solve kernels (cholesky.cu,
+// Pieces shared by the factorisation and solve kernels (cholesky.cu, chol_solve.cu,
 // chol_f64.cu): the counters of the task graph and the bounded waits on
 // them, 64x64 tile moves and products, and the factorisation of a diagonal
 // tile by one block.
