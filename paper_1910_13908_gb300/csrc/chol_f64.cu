@@ -285,6 +285,7 @@ __device__ void walker64_loads(const double* A, size_t lda, int n, const Sync64&
     bool ok = true;
     if (lane < 2) ok = wait_ge(sv.upd + (j + 1) * n + j + lane, j, status);
     ok = __all_sync(0xffffffffu, ok);
+    __syncwarp();  // a vote orders no memory: the other lanes' reads come after the acquire loads of lanes 0 and 1
     if (ok) {
       const double* Ap = A + ((size_t)(j + 1) * lda + j) * kNB64;
       double* d = W.diag[(j + 1) & 1];
