@@ -20,8 +20,9 @@
 // So every tile a claimed task waits for is written by a task claimed
 // before it or by the walker, and the walker waits only for tasks that
 // open once what it has published is published: some claimed task can
-// always run, whatever the number of blocks.  Every wait is bounded and
-// reports SC_STATUS_TIMEOUT.
+// always run, with one block beside the walker or more (the host launches two
+// at least, and at most half of the others leave the walker's SM,
+// LeaveWalkerSm).  Every wait is bounded and reports SC_STATUS_TIMEOUT.
 //
 // A batch of G jobs is one launch of G such sets of blocks.  A tile is
 // formed by the same operations whichever block forms it, so a job's factor
@@ -393,11 +394,9 @@ __global__ void __launch_bounds__(kBlock64) k_chol64(double* __restrict__ A0, in
   __shared__ Claim s_claim;
   __shared__ int s_first;
   const int tid = threadIdx.x, warp = tid >> 5;
-  int my_sm;
-  asm volatile("mov.u32 %0, %%smid;" : "=r"(my_sm));
   if (tid == 0) {
     s_first = atomicAdd(sv.fctr, 1) == 0;  // the first block to arrive
-    if (s_first) st_release(sv.sctr, my_sm + 1);
+    if (s_first) LeaveWalkerSm::publish(sv.sctr);
     W.failed = 0;
   }
   __syncthreads();
@@ -408,15 +407,16 @@ __global__ void __launch_bounds__(kBlock64) k_chol64(double* __restrict__ A0, in
     return;
   }
   if (warp >= kThr / 32) return;
-  // With blocks on several SMs, those that share the walker's leave it: the
-  // chain is the factorisation's critical path, and one warp instruction of
-  // theirs is 64 cycles of its.
+  // With blocks on several SMs, those that share the walker's leave it, up to
+  // half of them: one warp instruction of theirs is 64 cycles of its.
   const bool yield = per_job > 16 && (int)gridDim.x == per_job;
+  LeaveWalkerSm leave;
   int jp = 0, jb = 0;
   for (;;) {
     if (warp == 0) {
       Claim c = {-1, 0, 0, 0};
-      if (!(yield && ld_relaxed(sv.sctr) == my_sm + 1)) c = claim64(n, sv, status, jp, jb);
+      const int stay = __shfl_sync(0xffffffffu, !(yield && tid == 0 && leave.ask(sv.sctr, per_job)), 0);
+      if (stay) c = claim64(n, sv, status, jp, jb);
       if (tid == 0) s_claim = c;
     }
     csync();

@@ -12,8 +12,8 @@ namespace sc {
 
 enum TaskType { T_POTRF = 0, T_TRSM = 1, T_UPD = 2, T_FWD = 3, T_BWD = 4 };
 
-// sync area (ints): [0] factor task counter, [1] solve task counter (and,
-// during a factorisation, the walker's SM + 1), upd[nT*nT], potrf_done[nT],
+// sync area (ints): [0] factor task counter, [1] solve task counter (during a
+// factorisation LeaveWalkerSm's word), upd[nT*nT], potrf_done[nT],
 // trsm_done[nT*nT].  The solves pass their blocks as tagged words instead.
 struct SyncView {
   int* fctr;
@@ -69,6 +69,34 @@ static __device__ bool wait_ge(const int* p, int v, uint32_t* status) {
   atomicOr(status, SC_STATUS_TIMEOUT);
   return false;
 }
+
+// Blocks of a factorisation that share the walker's SM leave it to the
+// walker, which runs the critical path.  Not all of them may: every block can
+// land on that SM (the caller caps them to a few; or kernels of other streams
+// hold the rest of the GPU, and queued blocks come in one after another
+// through the slot the last one left), and the walker waits for tasks that
+// the others run.  So at most half of them leave, which is more than ever
+// share an SM with the walker when the blocks fill the GPU.
+__host__ __device__ constexpr int max_leavers(int blocks) { return (blocks - 1) / 2; }
+// Asked by one thread of a block before each claim.  `word`, the solve counter,
+// idle during a factorisation: the walker's SM + 1 (low half, stored once by
+// the walker) and the blocks that have asked to leave (high half).
+struct LeaveWalkerSm {
+  int state = 0;  // 1 stays, 2 leaves, 0 not known yet
+  __device__ __forceinline__ static int sm() {
+    int v;
+    asm volatile("mov.u32 %0, %%smid;" : "=r"(v));
+    return v;
+  }
+  __device__ __forceinline__ static void publish(int* word) { st_release(word, sm() + 1); }
+  __device__ __forceinline__ bool ask(int* word, int blocks) {
+    if (state == 0) {
+      const int w = ld_relaxed(word) & 0xffff;
+      if (w != 0) state = w == sm() + 1 && (atomicAdd(word, 1 << 16) >> 16) < max_leavers(blocks) ? 2 : 1;
+    }
+    return state == 2;
+  }
+};
 
 // mbarriers in shared memory
 namespace tc {

@@ -365,17 +365,10 @@ __global__ void __launch_bounds__(kCholThreads) k_chol(R* __restrict__ A, int ld
   SyncView sv(sync, nT);
   const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
   int next = -1;  // thread 0: the claimed, not yet examined task
-  // The walker publishes its SM (+1) in the otherwise idle solve counter; a
-  // block sharing that SM stops claiming, finishes what it holds and
-  // leaves the SM to the critical path.  A hint only: nothing depends on it.
-  int walker_sm = -1, my_sm = 0;
-  if (threadIdx.x == 0) asm volatile("mov.u32 %0, %%smid;" : "=r"(my_sm));
+  // a block that leaves the walker's SM stops claiming and finishes what it holds
+  LeaveWalkerSm leave;
   auto claim = [&]() -> int {  // thread 0
-    if (walker_sm < 0) {
-      const int w = ld_relaxed(sv.sctr);
-      if (w > 0) walker_sm = w - 1;
-    }
-    return walker_sm == my_sm ? n_tasks : atomicAdd(sv.fctr, 1);
+    return leave.ask(sv.sctr, gridDim.x) ? n_tasks : atomicAdd(sv.fctr, 1);
   };
   int4 cur = make_int4(-1, 0, 0, 0);
   bool have = false;  // cur's operands are queued in buffer pair buf
@@ -393,7 +386,7 @@ __global__ void __launch_bounds__(kCholThreads) k_chol(R* __restrict__ A, int ld
       const int t = s_task;
       if (t >= n_tasks) break;
       if (t == 0) {
-        if (threadIdx.x == 0) st_release(sv.sctr, my_sm + 1);
+        if (threadIdx.x == 0) LeaveWalkerSm::publish(sv.sctr);
         chol_walker(A, lda, nT, Linv, sv, status, lm, s0, s1, s2, aux, &s_bad, &s_ok);
         break;
       }
@@ -747,14 +740,9 @@ __global__ void __launch_bounds__(kCholThreads, 2) k_chol_tc(const __grid_consta
   uint32_t ph_load[2] = {0, 0}, ph_mma = 0;
   bool pend_load[2] = {false, false}, pend_mma = false;
   SyncView sv(sync, nT);
-  int walker_sm = -1, my_sm = 0;
-  if (threadIdx.x == 0) asm volatile("mov.u32 %0, %%smid;" : "=r"(my_sm));
+  LeaveWalkerSm leave;
   auto claim = [&]() -> int {  // thread 0
-    if (walker_sm < 0) {
-      const int w = ld_relaxed(sv.sctr);
-      if (w > 0) walker_sm = w - 1;
-    }
-    return walker_sm == my_sm ? n_tasks : atomicAdd(sv.fctr, 1);
+    return leave.ask(sv.sctr, gridDim.x) ? n_tasks : atomicAdd(sv.fctr, 1);
   };
   // thread 0: the operands of task tk into stage stg
   auto issue = [&](int4 tk, int stg) {
@@ -794,7 +782,7 @@ __global__ void __launch_bounds__(kCholThreads, 2) k_chol_tc(const __grid_consta
       const int t = ctl[0];
       if (t >= n_tasks) break;
       if (t == 0) {
-        if (threadIdx.x == 0) st_release(sv.sctr, my_sm + 1);
+        if (threadIdx.x == 0) LeaveWalkerSm::publish(sv.sctr);
         chol_walker(A, lda, nT, Linv, sv, status, lm, T0, T1, T2, aux, ctl + 2, ctl + 1);
         break;
       }
