@@ -989,6 +989,14 @@ static int chol_tc_grid() {
   return cached;
 }
 
+// Blocks of a factorisation with a walker, of at most `most` and the caller's
+// cap (0: none).  From three tile rows on the walker waits for tiles of
+// others, so it gets one block beside it whatever the cap.
+static int walker_grid(int most, int nT, int max_ctas) {
+  const int grid = std::min(most, chol_ntasks(nT));
+  return max_ctas > 0 ? std::max(std::min(grid, max_ctas), nT > 2 ? 2 : 1) : grid;
+}
+
 static cudaError_t launch_chol_tc(float* A, int lda, int nT, float* Linv, int* sync, uint32_t* status, LMState* lm,
                                   int max_ctas, cudaStream_t st, bool zeroed) {
   const int n_tasks = chol_ntasks(nT);
@@ -997,8 +1005,7 @@ static cudaError_t launch_chol_tc(float* A, int lda, int nT, float* Linv, int* s
   if (e != cudaSuccess) return e;
   e = encode_tile_map(&tmL, Linv, kNB, (uint64_t)nT * kNB, kNB * sizeof(float));
   if (e != cudaSuccess) return e;
-  int grid = std::min(chol_tc_grid(), n_tasks);
-  if (max_ctas > 0) grid = std::min(grid, max_ctas);
+  const int grid = walker_grid(chol_tc_grid(), nT, max_ctas);
   if (!zeroed) e = cudaMemsetAsync(sync, 0, sizeof(int) * chol_factor_reset_ints(nT), st);
   if (e != cudaSuccess) return e;
   return launch_dep(true, k_chol_tc, grid, kCholThreads, chol_tc_smem(), st, tmA, tmL, A, lda, nT, Linv, n_tasks, sync, status,
@@ -1015,8 +1022,7 @@ cudaError_t launch_chol(R* A, int lda, int nT, R* Linv, int* sync, uint32_t* sta
     int n_tasks = chol_ntasks(nT);
     size_t smem = sizeof(R) * (4 * kNB) * Pitch<R>::value;  // two buffer pairs; the walker uses 3.5 tiles
     const void* fn = reinterpret_cast<const void*>(&k_chol<R>);
-    int grid = std::min(chol_grid<R>(fn, smem), n_tasks);
-    if (max_ctas > 0) grid = std::min(grid, max_ctas);
+    const int grid = walker_grid(chol_grid<R>(fn, smem), nT, max_ctas);
     cudaError_t e = zeroed ? cudaSuccess : cudaMemsetAsync(sync, 0, sizeof(int) * chol_factor_reset_ints(nT), st);
     if (e != cudaSuccess) return e;
     return launch_dep(true, k_chol<R>, grid, kCholThreads, smem, st, A, lda, nT, Linv, n_tasks, sync, status, lm);

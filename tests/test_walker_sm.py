@@ -7,7 +7,8 @@ that other blocks run, so one of them has to stay.
 
 On the GPU: a calibration with the factorisation capped to a few blocks, where
 two or three can land on one SM, gives the bits of the one without a cap (a
-tile is formed by the same operations whichever block forms it).
+tile is formed by the same operations whichever block forms it).  A cap of
+one block counts as two: the walker alone would wait for tiles of others.
 """
 import os
 import re
@@ -45,7 +46,7 @@ def test_both_factorisations_ask_before_a_claim():
 
 
 @pytest.mark.gpu
-@pytest.mark.parametrize("max_ctas", [2, 3, 5, 17, 40])
+@pytest.mark.parametrize("max_ctas", [1, 2, 3, 5, 17, 40])
 @pytest.mark.parametrize("prec,kernel", [("mixed", 0), ("mixed", 1), ("fp64", 0)])
 def test_few_blocks_give_the_bits_of_many(prec, kernel, max_ctas):
     torch = pytest.importorskip("torch")
