@@ -81,12 +81,25 @@ __device__ __forceinline__ void tri_entry(int t, int& r, int& c) {
   else r = p, c = q - (16 - p);
 }
 
-// Reciprocal: the hardware's approximation (about 2^-20) and one step of third order.
-__device__ __forceinline__ double rcp64(double p) {
+// u / p for a pivot p > 0.  The reciprocal is the hardware's approximation
+// (about 2^-20) and one step of Halley's iteration, 1 / p = r / (1 - e) with
+// e = 1 - p r, taken as r (1 + e + e^2): off by e^3, below the roundings.  The
+// approximation flushes subnormal pivots and subnormal reciprocals to zero, so
+// below 2^-1022 and from 2^1022 on both numbers are first scaled by a power of
+// two (u <= sqrt(p A_rr) keeps the product in range; what underflows of u has
+// an underflowing quotient).
+__device__ __forceinline__ double over_pivot(double u, double p) {
+  const unsigned field = (unsigned)(__double2hiint(p) >> 20);  // the biased exponent; on the bits, off the float64 pipe
+  if (field - 1u >= 2044u) {
+    if (field == 0x7ff) return u * 0.0;  // p infinite
+    const double s = field == 0 ? 0x1p600 : 0x1p-600;
+    u *= s;
+    p *= s;
+  }
   double r;
   asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(p));
   const double e = fma(-p, r, 1.0);
-  return fma(r, fma(e, e, e), r);
+  return u * fma(r, fma(e, e, e), r);
 }
 
 struct Potrf64 {
@@ -124,7 +137,7 @@ __device__ bool potrf64(double* sm, double* sv, Potrf64& S) {
       p = 1.0;
       bad = true;
     }
-    const double cr = ur * rcp64(p);
+    const double cr = over_pivot(ur, p);
     const double ce = __shfl_sync(0xffffffffu, cr, row_lane);
     if (c == k && r > k) {
       S.u[r][k] = ur;
