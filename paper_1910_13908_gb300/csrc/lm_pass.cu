@@ -249,34 +249,60 @@ cudaError_t launch_sum_cost(const double* cpart, int N, double* out, cudaStream_
   return cudaGetLastError();
 }
 
-// Sum of n values by one block.  Float32 values are added as unevaluated
-// pairs hi + lo (TwoSum, six float32 additions, exact to about 2^-48): with
-// float64 additions, 16 cycles of an SM's pipe per warp, the block took 18 us
-// for the 2016 x 10 sums of 64 stations, now 10.
+// Sum of n values by one cluster.  Float32 values are added as unevaluated
+// triples hi + lo + tail (Ogita, Rump & Oishi 2005, SumK with K = 3): the
+// rounding errors of hi go to lo exactly and those of lo to tail, so a thread's
+// sum is off by its roundings to float64 and at most n_thread^2 2^-72.  What
+// bounds it is the issue of these 13 additions (float64 additions take 16
+// cycles of an SM's pipe per warp), which eight SMs share; a block's sum goes to
+// the first one's shared memory.  2016 x 10 values (64 stations) 7.7 us, 130816 x
+// 10 (512) 12.7; on one block 8.8 and 53.
+constexpr int kSumCtas = 8;
+__device__ __forceinline__ float two_sum(float a, float b, float& err) {  // a + b = result + err exactly
+  const float s = __fadd_rn(a, b), t = __fsub_rn(s, a);
+  err = __fadd_rn(__fsub_rn(a, __fsub_rn(s, t)), __fsub_rn(b, t));
+  return s;
+}
 template <typename R>
-__global__ void __launch_bounds__(1024) k_sum_reals(const R* __restrict__ x, int64_t n, double* __restrict__ out) {
-  __shared__ double sh[32];
+__global__ void __cluster_dims__(kSumCtas, 1, 1) __launch_bounds__(1024) k_sum_reals(const R* __restrict__ x, int64_t n,
+                                                                                    double* __restrict__ out) {
+  __shared__ double sh[32], s_part[kSumCtas];
+  asm volatile("barrier.cluster.arrive.release;" ::: "memory");  // waited for below: every block runs
+  const int64_t i0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, step = (int64_t)kSumCtas * blockDim.x;
   double a = 0.0;
+  bool add64 = true;
   if constexpr (sizeof(R) == 4) {
-    float hi = 0.f, lo = 0.f;
+    float hi = 0.f, lo = 0.f, tail = 0.f;
 #pragma unroll 8
-    for (int64_t i = threadIdx.x; i < n; i += blockDim.x) {
-      const float v = __ldg(x + i), s = __fadd_rn(hi, v), t = __fsub_rn(s, hi);
-      lo = __fadd_rn(lo, __fadd_rn(__fsub_rn(hi, __fsub_rn(s, t)), __fsub_rn(v, t)));
-      hi = s;
+    for (int64_t i = i0; i < n; i += step) {
+      float e, e2;
+      hi = two_sum(hi, __ldg(x + i), e);
+      lo = two_sum(lo, e, e2);
+      tail = __fadd_rn(tail, e2);
     }
-    a = (double)hi + (double)lo;
-    if (isfinite(hi)) n = 0;  // beyond float32's range: in float64 after all
-    else a = 0.0;
+    add64 = !isfinite(hi);  // beyond float32's range: in float64 after all
+    if (!add64) a = (double)hi + ((double)lo + (double)tail);
   }
-  for (int64_t i = threadIdx.x; i < n; i += blockDim.x) a += (double)x[i];
+  if (add64)
+    for (int64_t i = i0; i < n; i += step) a += (double)x[i];
   a = block_sum(a, sh);
-  if (threadIdx.x == 0) *out = a;
+  asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
+  if (threadIdx.x == 0) {
+    uint32_t dst;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, 0;" : "=r"(dst) : "r"((uint32_t)__cvta_generic_to_shared(s_part + blockIdx.x)));
+    asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(dst), "d"(a) : "memory");
+  }
+  asm volatile("barrier.cluster.arrive.release;\n barrier.cluster.wait.acquire;" ::: "memory");
+  if (blockIdx.x == 0 && threadIdx.x == 0) {
+    double t = 0.0;
+    for (int c = 0; c < kSumCtas; ++c) t += s_part[c];
+    *out = t;
+  }
 }
 
 template <typename R>
 cudaError_t launch_sum_reals(const R* x, int64_t n, double* out, cudaStream_t st) {
-  k_sum_reals<R><<<1, 1024, 0, st>>>(x, n, out);
+  k_sum_reals<R><<<kSumCtas, 1024, 0, st>>>(x, n, out);
   return cudaGetLastError();
 }
 template cudaError_t launch_sum_reals<float>(const float*, int64_t, double*, cudaStream_t);
