@@ -151,10 +151,13 @@ typedef struct sc_lm_opts {
   double eps_grad;       /* stop once max|J^T r| <= eps_grad * (1 + cost) */
   int32_t max_ctas;      /* cap on the thread blocks of the persistent
                             factorisation kernel; 0 = enough to fill the GPU.
-                            Lower it when several jobs share the device.  The
-                            block on the diagonal chain has at least one more
-                            beside it: a cap of 1 counts as 2 (in SC_FP64 as 2
-                            for each job of a batch) */
+                            Set it when several jobs share the device: a job
+                            with a cap also solves without thread-block
+                            clusters, which wait long for free multiprocessors
+                            beside other jobs (the same results).  The block
+                            on the diagonal chain has at least one more beside
+                            it: a cap of 1 counts as 2 (in SC_FP64 as 2 for
+                            each job of a batch) */
   int32_t chol_kernel;   /* SC_MIXED: which factorisation kernel runs the
                             64x64 tile products of the bulk,
                             SC_CHOL_SIMT (0, the default) or SC_CHOL_TENSOR

@@ -328,6 +328,7 @@ static int lm_solve(const Ctx& c, const R* Xin, bool running, const R* C, const 
   uint64_t* bw = c.at<uint64_t>(L.bvec);
   int* sync = c.at<int>(L.sync);
   const int n_sync = chol_sync_ints(L.nT, s.prec);
+  const bool shared = o.max_ctas > 0;  // a cap: other jobs run beside this one
   LMState* lm = c.lm();
 
   SC_CUDA(cudaMemcpyAsync(J_old, J_io, n8, cudaMemcpyDeviceToDevice, c.st));
@@ -345,12 +346,12 @@ static int lm_solve(const Ctx& c, const R* Xin, bool running, const R* C, const 
     SC_LAUNCH(PK_ASSEMBLE, launch_assemble<R>(s, L.Ppad, L.Ppad, w, Jr, b.H_cur, lm, A, true, false, c.st, Batch{}, sync,
                                               n_sync));
     SC_LAUNCH(PK_CHOL, launch_chol<R>(A, L.Ppad, L.nT, Linv, sync, c.status(), lm, o.max_ctas, o.chol_kernel, c.st, true));
-    SC_LAUNCH(PK_SOLVE, launch_chol_solve<R>(A, L.Ppad, L.nT, Linv, sync, b.g_cur, bw, x, 0, c.status(), lm, c.st));
+    SC_LAUNCH(PK_SOLVE, launch_chol_solve<R>(A, L.Ppad, L.nT, Linv, sync, b.g_cur, bw, x, 0, c.status(), lm, c.st, shared));
     if (mixed) {
       for (int sw = 0; sw < o.refine_sweeps; ++sw) {
         SC_LAUNCH(PK_REFINE, launch_refine_residual<R>(s, w, b.J_cur, b.H_cur, b.g_cur, x, lm, c.at<double>(L.ry),
                                                        rvec, c.st));
-        SC_LAUNCH(PK_SOLVE, launch_chol_solve<R>(A, L.Ppad, L.nT, Linv, sync, rvec, bw, x, 1, c.status(), lm, c.st));
+        SC_LAUNCH(PK_SOLVE, launch_chol_solve<R>(A, L.Ppad, L.nT, Linv, sync, rvec, bw, x, 1, c.status(), lm, c.st, shared));
       }
     }
     SC_LAUNCH(PK_LM, launch_lm_trial(lm, s.N, x, b, c.st));
@@ -601,6 +602,7 @@ static int sage_batched(const Ctx& c, const std::vector<Ctx>& jc, const sc_job* 
   uint64_t* bw = c.at<uint64_t>(L.bvec);
   int* sync = c.at<int>(L.sync);
   const int n_sync = chol_sync_ints(L.nT, s.prec);
+  const bool shared = o.lm.max_ctas > 0;  // a cap: other jobs run beside the batch
   LMState* lm = c.lm();
   const int* nchunk_dev = &lm->nchunk;
   auto blk = [&](int g) { return c.base + (size_t)g * js; };
@@ -652,13 +654,13 @@ static int sage_batched(const Ctx& c, const std::vector<Ctx>& jc, const sc_job* 
         SC_LAUNCH(PK_CHOL, launch_chol_batch<R>(A, L.Ppad, L.nT, Linv, sync, c.status(), lm, o.lm.max_ctas, bt,
                                                 order, c.st, true));
         SC_LAUNCH(PK_SOLVE, launch_chol_solve<R>(A, L.Ppad, L.nT, Linv, sync, b.g_cur, bw, x, 0, c.status(), lm,
-                                                 c.st, bt));
+                                                 c.st, shared, bt));
         if (mixed) {
           for (int sw = 0; sw < o.lm.refine_sweeps; ++sw) {
             SC_LAUNCH(PK_REFINE, launch_refine_residual<R>(s, w, b.J_cur, b.H_cur, b.g_cur, x, lm,
                                                            c.at<double>(L.ry), rvec, c.st, bt));
             SC_LAUNCH(PK_SOLVE, launch_chol_solve<R>(A, L.Ppad, L.nT, Linv, sync, rvec, bw, x, 1, c.status(), lm,
-                                                     c.st, bt));
+                                                     c.st, shared, bt));
           }
         }
         SC_LAUNCH(PK_LM, launch_lm_trial(lm, s.N, x, b, c.st, bt));
@@ -885,7 +887,7 @@ static int cholesky_impl(int n, R* A, int lda, const double* b, double* x, int k
     SC_CUDA(cudaMemcpyAsync(bpad, b, (size_t)n * 8, cudaMemcpyDeviceToDevice, st));
     SC_CUDA(cudaMemsetAsync(bw, 0, (size_t)L.Ppad * 2 * sizeof(R), st));
     prof_start(PK_SOLVE, st);
-    const cudaError_t se = launch_chol_solve<R>(Aw, L.Ppad, L.nT, Linv, sync, bpad, bw, xpad, 0, status, nullptr, st);
+    const cudaError_t se = launch_chol_solve<R>(Aw, L.Ppad, L.nT, Linv, sync, bpad, bw, xpad, 0, status, nullptr, st, false);
     prof_stop(PK_SOLVE, st);
     SC_CUDA(se);
     SC_CUDA(cudaMemcpyAsync(x, xpad, (size_t)n * 8, cudaMemcpyDeviceToDevice, st));
@@ -1169,7 +1171,8 @@ SC_API int32_t sc_calibrate_batch(const sc_job* jobs, int32_t n_jobs, const sc_s
   unsigned hw = std::max(1u, std::thread::hardware_concurrency());
   int workers = (int)std::min<unsigned>((unsigned)n_jobs, std::min(hw, 16u));
   sc_sage_opts o = *opts;
-  if (o.lm.max_ctas == 0) o.lm.max_ctas = std::max(8, 2 * sms / workers);
+  // a cap also says that jobs share the device: none for a job alone
+  if (o.lm.max_ctas == 0 && n_jobs > 1) o.lm.max_ctas = std::max(8, 2 * sms / workers);
   std::atomic<int> next{0};
   std::atomic<int> first_err{0};
   std::vector<std::string> msgs(workers);

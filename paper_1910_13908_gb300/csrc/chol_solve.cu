@@ -415,9 +415,14 @@ int resident_clusters(int nc) {
 // 8 CTAs up to 8 tile rows, else 16 where the device takes such clusters (one
 // row per CTA keeps a block's products ahead of the chain).  A batch goes to
 // k_chol_solve once its clusters would not all be resident: its rows then fill
-// the GPU without them.
-int solve_cluster_size(int nT, int G) {
-  if (nT < 2 || nT > kMaxRows) return 0;
+// the GPU without them.  So does a job that shares the device: a cluster starts
+// only once 8 or 16 SMs of one GPC have 187 KB of shared memory free at the same
+// time, and waits long for that while factorisations of other streams come and
+// go.  Jobs on 16 streams, k_chol_solve against clusters: 32 jobs of 64 stations
+// 29 ms, 37; 24 of 128 stations 52, 89; alone a solve of 64 stations takes 23.9
+// us, 17.5.
+int solve_cluster_size(int nT, int G, bool shared) {
+  if (shared || nT < 2 || nT > kMaxRows) return 0;
   // per device: 1 + the resident clusters of 8 and of 16 CTAs (0: not asked yet)
   constexpr int kDevs = 64;
   static std::atomic<int> cache[2][kDevs];

@@ -419,8 +419,9 @@ cudaError_t launch_solve64(const double* A, int lda, int nT, const double* Linv,
                            const LMState* lm, cudaStream_t st, const Batch& bt = Batch{});
 int chol64_b_task(int n, int j, int idx, int* I, int* K);
 // CTAs of the cluster that solves one of G float32 systems of nT tile rows
-// (0: k_chol_solve takes the call), and that solve.
-int solve_cluster_size(int nT, int G);
+// (0: k_chol_solve takes the call), and that solve.  shared: other jobs run on
+// the device at the same time.
+int solve_cluster_size(int nT, int G, bool shared);
 cudaError_t launch_chol_solve_cluster(const float* A, int lda, int nT, int nc, const float* Linv, const double* b,
                                       double* x, int accumulate, uint32_t* status, const LMState* lm, cudaStream_t st,
                                       const Batch& bt);
@@ -441,7 +442,8 @@ cudaError_t launch_batch_order(int nT, int G, int W, uint32_t* order, cudaStream
 template <typename R>
 cudaError_t launch_chol_solve(const R* A, int lda, int nT, const R* Linv, int* sync,
                               const double* b, uint64_t* bwork, double* x, int accumulate,
-                              uint32_t* status, const LMState* lm, cudaStream_t st, const Batch& bt = Batch{});
+                              uint32_t* status, const LMState* lm, cudaStream_t st, bool shared,
+                              const Batch& bt = Batch{});
 
 // lm_control.cu
 cudaError_t launch_lm_init(LMState* lm, const sc_lm_opts* o, int N, const LMBufs& b, const double* J_src,

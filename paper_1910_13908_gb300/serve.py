@@ -322,6 +322,8 @@ class Server(Scheduler):
             free, _ = torch.cuda.mem_get_info(dev)
             mem_budget = int(0.8 * free)
         max_ctas = max(8, 2 * torch.cuda.get_device_properties(dev).multi_processor_count // max_slots)
+        if max_slots == 1:  # one job at a time: the whole device
+            max_ctas = 0
         super().__init__(CudaBackend(prec, device, n_em, n_lm, refine_sweeps, max_ctas, enqueue_threads),
                          mem_budget, max_slots)
         self.prec = prec
