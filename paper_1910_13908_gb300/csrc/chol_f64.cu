@@ -219,7 +219,7 @@ __host__ __device__ __forceinline__ int b_count64(int n, int j) {
   return m * (m + 1) / 2;
 }
 // B task idx of panel j: pairs (I, K), column pair by column pair
-__host__ __device__ __forceinline__ void b_task64(int n, int j, int idx, int& I, int& K) {
+__device__ __forceinline__ void b_task64(int n, int j, int idx, int& I, int& K) {
   const int m = b_first64(n, j);
   // pairs before x hold x m - x (x - 1) / 2 tasks
   const float h = m + 0.5f;
@@ -748,13 +748,6 @@ cudaError_t launch_solve64(const double* A, int lda, int nT, const double* Linv,
   if (e != cudaSuccess) return e;
   return launch_dep(bt.js == 0, k_solve64, 2 * nS * bt.G, kThr, 0, st, A, lda, nS, Linv, sync, b, bwork, x, accumulate, tag, status,
                     lm, bt.G, bt.js);
-}
-
-// Host view of the enumeration: B task idx of panel j of n tiles as (I, K);
-// the number of B tasks when idx < 0.
-int chol64_b_task(int n, int j, int idx, int* I, int* K) {
-  if (idx >= 0) b_task64(n, j, idx, *I, *K);
-  return b_count64(n, j);
 }
 
 }  // namespace sc

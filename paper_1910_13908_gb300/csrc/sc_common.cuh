@@ -417,7 +417,6 @@ cudaError_t launch_chol64(double* A, int lda, int nT, double* Linv, int* sync, u
 cudaError_t launch_solve64(const double* A, int lda, int nT, const double* Linv, int* sync, const double* b,
                            uint64_t* bwork, double* x, int accumulate, uint32_t tag, uint32_t* status,
                            const LMState* lm, cudaStream_t st, const Batch& bt = Batch{});
-int chol64_b_task(int n, int j, int idx, int* I, int* K);
 // CTAs of the cluster that solves one of G float32 systems of nT tile rows
 // (0: k_chol_solve takes the call), and that solve.  shared: other jobs run on
 // the device at the same time.
