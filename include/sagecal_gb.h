@@ -154,7 +154,8 @@ typedef struct sc_lm_opts {
                             Set it when several jobs share the device: a job
                             with a cap also solves without thread-block
                             clusters, which wait long for free multiprocessors
-                            beside other jobs (the same results).  The block
+                            beside other jobs (the same results; the bands of
+                            one consensus call keep them).  The block
                             on the diagonal chain has at least one more beside
                             it: a cap of 1 counts as 2 (in SC_FP64 as 2 for
                             each job of a batch) */

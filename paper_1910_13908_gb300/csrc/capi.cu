@@ -160,6 +160,7 @@ struct Ctx {
   char* base;
   cudaStream_t st;
   int splits;  // ranges of the float32 sums w_pq
+  bool bands = false;  // one of several bands calibrated at once
   template <class T>
   T* at(size_t off) const {
     return reinterpret_cast<T*>(base + off);
@@ -328,7 +329,8 @@ static int lm_solve(const Ctx& c, const R* Xin, bool running, const R* C, const 
   uint64_t* bw = c.at<uint64_t>(L.bvec);
   int* sync = c.at<int>(L.sync);
   const int n_sync = chol_sync_ints(L.nT, s.prec);
-  const bool shared = o.max_ctas > 0;  // a cap: other jobs run beside this one
+  // a cap says that other jobs share the device
+  const Beside beside = c.bands ? Beside::bands : o.max_ctas > 0 ? Beside::jobs : Beside::nothing;
   LMState* lm = c.lm();
 
   SC_CUDA(cudaMemcpyAsync(J_old, J_io, n8, cudaMemcpyDeviceToDevice, c.st));
@@ -346,12 +348,12 @@ static int lm_solve(const Ctx& c, const R* Xin, bool running, const R* C, const 
     SC_LAUNCH(PK_ASSEMBLE, launch_assemble<R>(s, L.Ppad, L.Ppad, w, Jr, b.H_cur, lm, A, true, false, c.st, Batch{}, sync,
                                               n_sync));
     SC_LAUNCH(PK_CHOL, launch_chol<R>(A, L.Ppad, L.nT, Linv, sync, c.status(), lm, o.max_ctas, o.chol_kernel, c.st, true));
-    SC_LAUNCH(PK_SOLVE, launch_chol_solve<R>(A, L.Ppad, L.nT, Linv, sync, b.g_cur, bw, x, 0, c.status(), lm, c.st, shared));
+    SC_LAUNCH(PK_SOLVE, launch_chol_solve<R>(A, L.Ppad, L.nT, Linv, sync, b.g_cur, bw, x, 0, c.status(), lm, c.st, beside));
     if (mixed) {
       for (int sw = 0; sw < o.refine_sweeps; ++sw) {
         SC_LAUNCH(PK_REFINE, launch_refine_residual<R>(s, w, b.J_cur, b.H_cur, b.g_cur, x, lm, c.at<double>(L.ry),
                                                        rvec, c.st));
-        SC_LAUNCH(PK_SOLVE, launch_chol_solve<R>(A, L.Ppad, L.nT, Linv, sync, rvec, bw, x, 1, c.status(), lm, c.st, shared));
+        SC_LAUNCH(PK_SOLVE, launch_chol_solve<R>(A, L.Ppad, L.nT, Linv, sync, rvec, bw, x, 1, c.status(), lm, c.st, beside));
       }
     }
     SC_LAUNCH(PK_LM, launch_lm_trial(lm, s.N, x, b, c.st));
@@ -602,7 +604,7 @@ static int sage_batched(const Ctx& c, const std::vector<Ctx>& jc, const sc_job* 
   uint64_t* bw = c.at<uint64_t>(L.bvec);
   int* sync = c.at<int>(L.sync);
   const int n_sync = chol_sync_ints(L.nT, s.prec);
-  const bool shared = o.lm.max_ctas > 0;  // a cap: other jobs run beside the batch
+  const Beside beside = o.lm.max_ctas > 0 ? Beside::jobs : Beside::nothing;
   LMState* lm = c.lm();
   const int* nchunk_dev = &lm->nchunk;
   auto blk = [&](int g) { return c.base + (size_t)g * js; };
@@ -654,13 +656,13 @@ static int sage_batched(const Ctx& c, const std::vector<Ctx>& jc, const sc_job* 
         SC_LAUNCH(PK_CHOL, launch_chol_batch<R>(A, L.Ppad, L.nT, Linv, sync, c.status(), lm, o.lm.max_ctas, bt,
                                                 order, c.st, true));
         SC_LAUNCH(PK_SOLVE, launch_chol_solve<R>(A, L.Ppad, L.nT, Linv, sync, b.g_cur, bw, x, 0, c.status(), lm,
-                                                 c.st, shared, bt));
+                                                 c.st, beside, bt));
         if (mixed) {
           for (int sw = 0; sw < o.lm.refine_sweeps; ++sw) {
             SC_LAUNCH(PK_REFINE, launch_refine_residual<R>(s, w, b.J_cur, b.H_cur, b.g_cur, x, lm,
                                                            c.at<double>(L.ry), rvec, c.st, bt));
             SC_LAUNCH(PK_SOLVE, launch_chol_solve<R>(A, L.Ppad, L.nT, Linv, sync, rvec, bw, x, 1, c.status(), lm,
-                                                     c.st, shared, bt));
+                                                     c.st, beside, bt));
           }
         }
         SC_LAUNCH(PK_LM, launch_lm_trial(lm, s.N, x, b, c.st, bt));
@@ -887,7 +889,7 @@ static int cholesky_impl(int n, R* A, int lda, const double* b, double* x, int k
     SC_CUDA(cudaMemcpyAsync(bpad, b, (size_t)n * 8, cudaMemcpyDeviceToDevice, st));
     SC_CUDA(cudaMemsetAsync(bw, 0, (size_t)L.Ppad * 2 * sizeof(R), st));
     prof_start(PK_SOLVE, st);
-    const cudaError_t se = launch_chol_solve<R>(Aw, L.Ppad, L.nT, Linv, sync, bpad, bw, xpad, 0, status, nullptr, st, false);
+    const cudaError_t se = launch_chol_solve<R>(Aw, L.Ppad, L.nT, Linv, sync, bpad, bw, xpad, 0, status, nullptr, st, Beside::nothing);
     prof_stop(PK_SOLVE, st);
     SC_CUDA(se);
     SC_CUDA(cudaMemcpyAsync(x, xpad, (size_t)n * 8, cudaMemcpyDeviceToDevice, st));
@@ -1118,6 +1120,7 @@ SC_API int32_t sc_calibrate_consensus(const sc_dims* d, int32_t n_bands, const d
     if (so.lm.max_ctas == 0) so.lm.max_ctas = std::max(8, 2 * device_sms() / m);
   }
   std::vector<Ctx> band(m, c);
+  for (Ctx& b : band) b.bands = m > 1;
   for (int k = 1; k < m; ++k) {
     band[k].base = c.base + per * k;
     SC_CUDA(cudaMemsetAsync(band[k].status(), 0, 256, c.st));

@@ -415,14 +415,21 @@ int resident_clusters(int nc) {
 // 8 CTAs up to 8 tile rows, else 16 where the device takes such clusters (one
 // row per CTA keeps a block's products ahead of the chain).  A batch goes to
 // k_chol_solve once its clusters would not all be resident: its rows then fill
-// the GPU without them.  So does a job that shares the device: a cluster starts
-// only once 8 or 16 SMs of one GPC have 187 KB of shared memory free at the same
-// time, and waits long for that while factorisations of other streams come and
-// go.  Jobs on 16 streams, k_chol_solve against clusters: 32 jobs of 64 stations
-// 29 ms, 37; 24 of 128 stations 52, 89; alone a solve of 64 stations takes 23.9
-// us, 17.5.
-int solve_cluster_size(int nT, int G, bool shared) {
-  if (shared || nT < 2 || nT > kMaxRows) return 0;
+// the GPU without them.
+//
+// Beside other work a cluster is slow to start: it waits until 8 or 16 SMs of
+// one GPC have 187 KB of shared memory free at the same time, while
+// factorisations of other streams come and go, and launched early it keeps
+// those SMs from them.  So a job whose factorisation the caller caps, which
+// says that other jobs share the device, goes to k_chol_solve; jobs on 16
+// streams, against clusters and against clusters launched the plain way: 32
+// jobs of 64 stations 29 ms, 37 and 30, 24 of 128 stations 52, 89 and 61.  The
+// bands of a consensus, which one host thread enqueues, leave SMs free: clusters
+// there too, those of 16 CTAs launched the plain way.  16 bands of 128 stations
+// and 10 clusters (16 CTAs) 221 ms, 296 launched early, 374 in k_chol_solve; of
+// 64 stations and 12 clusters (8 CTAs) 228, 216 and 314.
+int solve_cluster_size(int nT, int G, Beside beside) {
+  if (beside == Beside::jobs || nT < 2 || nT > kMaxRows) return 0;
   // per device: 1 + the resident clusters of 8 and of 16 CTAs (0: not asked yet)
   constexpr int kDevs = 64;
   static std::atomic<int> cache[2][kDevs];
@@ -439,7 +446,7 @@ int solve_cluster_size(int nT, int G, bool shared) {
 
 cudaError_t launch_chol_solve_cluster(const float* A, int lda, int nT, int nc, const float* Linv, const double* b,
                                       double* x, int accumulate, uint32_t* status, const LMState* lm, cudaStream_t st,
-                                      const Batch& bt) {
+                                      bool early, const Batch& bt) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(nc, bt.G, 1);
   cfg.blockDim = dim3(kThreads, 1, 1);
@@ -450,7 +457,7 @@ cudaError_t launch_chol_solve_cluster(const float* A, int lda, int nT, int nc, c
   at[0].val.clusterDim.x = nc;
   at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
   at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;  // as launch_dep
-  at[1].val.programmaticStreamSerializationAllowed = bt.js == 0;
+  at[1].val.programmaticStreamSerializationAllowed = early ? 1 : 0;
   cfg.attrs = at;
   cfg.numAttrs = 2;
   return cudaLaunchKernelEx(&cfg, k_chol_solve_cluster, A, lda, nT, Linv, b, x, accumulate, status, lm, bt.js);

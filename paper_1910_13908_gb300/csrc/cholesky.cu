@@ -1357,14 +1357,15 @@ static std::atomic<uint32_t> g_solve_launches{0};
 template <typename R>
 cudaError_t launch_chol_solve(const R* A, int lda, int nT, const R* Linv, int* sync,
                               const double* b, uint64_t* bwork, double* x, int accumulate,
-                              uint32_t* status, const LMState* lm, cudaStream_t st, bool shared, const Batch& bt) {
+                              uint32_t* status, const LMState* lm, cudaStream_t st, Beside beside, const Batch& bt) {
   // tags 2e (forward) and 2e + 1 (backward), e >= 1, unique per launch
   const uint32_t e = (g_solve_launches.fetch_add(1, std::memory_order_relaxed) % 0x7ffffffeu) + 1;
   if constexpr (sizeof(R) == 8) {
     return launch_solve64(A, lda, nT, Linv, sync, b, bwork, x, accumulate, 2 * e, status, lm, st, bt);
   } else {
-    if (const int nc = solve_cluster_size(nT, bt.G, shared))
-      return launch_chol_solve_cluster(A, lda, nT, nc, Linv, b, x, accumulate, status, lm, st, bt);
+    if (const int nc = solve_cluster_size(nT, bt.G, beside))
+      return launch_chol_solve_cluster(A, lda, nT, nc, Linv, b, x, accumulate, status, lm, st,
+                                       bt.js == 0 && (beside == Beside::nothing || nc == 8), bt);
     int n_tasks = 2 * nT;
     if ((long long)n_tasks * bt.G > (1LL << 30)) return cudaErrorInvalidValue;
     size_t smem = sizeof(R) * (4 * kNB * Pitch<R>::value + kNB);
@@ -1383,9 +1384,9 @@ cudaError_t launch_chol_solve(const R* A, int lda, int nT, const R* Linv, int* s
 }
 template cudaError_t launch_chol_solve<float>(const float*, int, int, const float*, int*,
                                               const double*, uint64_t*, double*, int, uint32_t*,
-                                              const LMState*, cudaStream_t, bool, const Batch&);
+                                              const LMState*, cudaStream_t, Beside, const Batch&);
 template cudaError_t launch_chol_solve<double>(const double*, int, int, const double*, int*,
                                                const double*, uint64_t*, double*, int, uint32_t*,
-                                               const LMState*, cudaStream_t, bool, const Batch&);
+                                               const LMState*, cudaStream_t, Beside, const Batch&);
 
 }  // namespace sc

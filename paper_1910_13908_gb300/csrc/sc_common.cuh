@@ -417,13 +417,14 @@ cudaError_t launch_chol64(double* A, int lda, int nT, double* Linv, int* sync, u
 cudaError_t launch_solve64(const double* A, int lda, int nT, const double* Linv, int* sync, const double* b,
                            uint64_t* bwork, double* x, int accumulate, uint32_t tag, uint32_t* status,
                            const LMState* lm, cudaStream_t st, const Batch& bt = Batch{});
+// What runs beside a job, for the choice of its float32 solve (solve_cluster_size).
+enum class Beside { nothing, bands, jobs };
 // CTAs of the cluster that solves one of G float32 systems of nT tile rows
-// (0: k_chol_solve takes the call), and that solve.  shared: other jobs run on
-// the device at the same time.
-int solve_cluster_size(int nT, int G, bool shared);
+// (0: k_chol_solve takes the call), and that solve.
+int solve_cluster_size(int nT, int G, Beside beside);
 cudaError_t launch_chol_solve_cluster(const float* A, int lda, int nT, int nc, const float* Linv, const double* b,
                                       double* x, int accumulate, uint32_t* status, const LMState* lm, cudaStream_t st,
-                                      const Batch& bt);
+                                      bool early, const Batch& bt);
 // The factorisations of a whole batch as one persistent launch: the task
 // lists of the G jobs interleaved (task t is task t / G of job t mod G), no
 // walker; every tile is computed by the same arithmetic as in launch_chol.
@@ -441,7 +442,7 @@ cudaError_t launch_batch_order(int nT, int G, int W, uint32_t* order, cudaStream
 template <typename R>
 cudaError_t launch_chol_solve(const R* A, int lda, int nT, const R* Linv, int* sync,
                               const double* b, uint64_t* bwork, double* x, int accumulate,
-                              uint32_t* status, const LMState* lm, cudaStream_t st, bool shared,
+                              uint32_t* status, const LMState* lm, cudaStream_t st, Beside beside,
                               const Batch& bt = Batch{});
 
 // lm_control.cu

@@ -2,8 +2,9 @@
 
 A thread-block cluster waits long for its multiprocessors while other streams'
 factorisations hold them, so a job whose factorisation is capped (the caller's
-max_ctas, a batch on streams, concurrent bands) solves without one.  The kernels
-that ran are read from the profiler's trace; the results are the same bits."""
+max_ctas, a batch on streams) solves without one; the bands of a consensus keep
+it.  The kernels that ran are read from the profiler's trace; the results are the
+same bits."""
 import pytest
 
 torch = pytest.importorskip("torch")
@@ -68,3 +69,21 @@ def test_jobs_on_streams(n_jobs, solver):
         _sage(j, 0)
         torch.cuda.synchronize()
         assert torch.equal(j.jones, jones) and torch.equal(j.costs, costs)
+
+
+def test_concurrent_bands_keep_the_cluster():
+    j, n_bands = _job(20), 3
+    freqs = (j.freqs + 1e6 * torch.arange(n_bands, device="cuda", dtype=torch.float64)[:, None]).contiguous()
+    V = j.V[None].repeat(n_bands, 1, 1, 1, 1, 1).contiguous()
+    basis = torch.ones((n_bands, 1), dtype=torch.float64, device="cuda")
+    out = {}
+
+    def consensus(concurrent):
+        jones = j.jones[None].repeat(n_bands, 1, 1, 1, 1).contiguous()
+        ws = sc.consensus_workspace(j.shape, sc.SC_MIXED, concurrent)
+        out[concurrent] = sc.calibrate_consensus(j.shape, j.uvw, freqs, j.sky, V, basis, jones, sc.SC_MIXED, ws, 1.0,
+                                                 n_admm=2, n_em=1, n_lm=3)
+
+    assert _solvers(lambda: consensus(n_bands)) == {"cluster"}
+    assert _solvers(lambda: consensus(1)) == {"cluster"}
+    assert all(torch.equal(a, b) for a, b in zip(out[n_bands], out[1]))
