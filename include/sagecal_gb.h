@@ -541,7 +541,8 @@ typedef struct sc_job {
  * GPU).  Each job is calibrated exactly as by sc_calibrate_sage on its own
  * stream with its own workspace; a pool of host threads enqueues them so
  * that they overlap on the device, and the factorisation kernel of each job
- * is capped (opts->lm.max_ctas, or an even share of the GPU when 0).  Results
+ * is capped (opts->lm.max_ctas, or an even share of the GPU when 0; a single
+ * job is not).  Results
  * of a job do not depend on the other jobs.  Returns when every job has been
  * enqueued; the first error (if any) is returned and later jobs are still
  * attempted.  The device takes the streams' launches through a fixed number
@@ -592,7 +593,8 @@ SC_API int32_t sc_calibrate_batched(const sc_job* jobs, int32_t n_jobs, const sc
  * (each in [1, 2^20]; one above (n_jobs - 1) x the tasks of one job
  * orders the tasks as the interleave does), times `reps` factorisations of the
  * jobs' matrix order (identity matrices: the arithmetic takes the same time
- * on any values) in the batch workspace ws (sc_batched_workspace_size of
+ * on any values; in SC_FP64 the order has no effect, and the times differ by
+ * noise) in the batch workspace ws (sc_batched_workspace_size of
  * dims), after one untimed run, with CUDA events on `stream`; writes the
  * mean milliseconds per factorisation to ms_out[n_windows] and the fastest
  * window to *best.  Synchronises `stream` (the one call of this library

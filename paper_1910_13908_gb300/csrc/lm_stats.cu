@@ -496,8 +496,8 @@ __device__ __forceinline__ void eval_baseline(const double* stat, int64_t B, int
 // entries of G are loops, the latter with the thread's numbers in shared memory,
 // and the next chunk's loads go out before the current one is added.  An LM
 // iteration of 64 stations (10 blocks, 10 chunks) 184 -> 175 us; a batch of 16
-// jobs of 256 (2176 blocks) is 0.4% faster the other way, at three blocks more
-// per SM.
+// jobs of 256 (2176 blocks) is 0.4% faster the other way, at 64 registers and
+// four blocks per SM instead of 100 and two.
 struct EvalBuf {
   float2 v[kStatV][kST * kST];  // rhoX and W, pairs
   float g[8][kST * kST];        // G, then rho

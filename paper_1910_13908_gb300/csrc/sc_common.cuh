@@ -149,8 +149,8 @@ __device__ __forceinline__ void bl_pair(int64_t b, int N, int& p, int& q) {
 // dep_sync, the first statement of every kernel launched that way, waits until
 // that kernel has completed and its stores are visible; only then may the
 // blocks of the kernel after this one come in, so at most one kernel waits in
-// place.  An iteration of 64 stations takes 192 us instead of 215, of 128 323
-// instead of 345.  A batch's launches and large assemblies, whose many short
+// place.  An iteration of 64 stations took 194 us instead of 215, of 128 323
+// instead of 345 (173 and 309 with what followed).  A batch's launches and large assemblies, whose many short
 // blocks the two instructions would slow down (batch of 64 jobs: 1.6%), go the
 // plain way: early is given to the kernel and to its launch alike.
 __device__ __forceinline__ void dep_sync(bool early) {
