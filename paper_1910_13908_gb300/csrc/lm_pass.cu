@@ -249,34 +249,38 @@ cudaError_t launch_sum_cost(const double* cpart, int N, double* out, cudaStream_
   return cudaGetLastError();
 }
 
-// Sum of n values by one cluster.  Float32 values are added as unevaluated
-// triples hi + lo + tail (Ogita, Rump & Oishi 2005, SumK with K = 3): the
-// rounding errors of hi go to lo exactly and those of lo to tail, so a thread's
-// sum is off by its roundings to float64 and at most n_thread^2 2^-72.  What
-// bounds it is the issue of these 13 additions (float64 additions take 16
-// cycles of an SM's pipe per warp), which eight SMs share; a block's sum goes to
-// the first one's shared memory.  2016 x 10 values (64 stations) 7.7 us, 130816 x
-// 10 (512) 12.7; on one block 8.8 and 53.
-constexpr int kSumCtas = 8;
+// Sum of n values.  Float32 values are added as unevaluated triples hi + lo +
+// tail (Ogita, Rump & Oishi 2005, SumK with K = 3): the rounding errors of hi go
+// to lo exactly and those of lo to tail, so a thread's sum is off by its roundings
+// to float64 and at most n_thread^2 2^-72.  What bounds it is the issue of these
+// 13 additions (float64 additions take 16 cycles of an SM's pipe per warp): up to
+// kSumOne values are one block's, more are cut into segments of a block each,
+// whose sums replace the first values of the segments, and a second kernel adds
+// them.  2016 x 10 values (64 stations) 8.4 us; 130816 x 3 (512 stations, 10
+// timeslots) 7.9 + 3.7, one block 53.  A cluster of eight blocks took 7.7 and 12.7
+// without the second kernel, but waited for its eight SMs beside other streams'
+// factorisations: the call's 90th percentile 1400 us instead of 200.
+constexpr int kSumThreads = 1024;
+constexpr int64_t kSumOne = 32768, kSumSegment = 8192;
+constexpr int kSumBlocks = 64;
 __device__ __forceinline__ float two_sum(float a, float b, float& err) {  // a + b = result + err exactly
   const float s = __fadd_rn(a, b), t = __fsub_rn(s, a);
   err = __fadd_rn(__fsub_rn(a, __fsub_rn(s, t)), __fsub_rn(b, t));
   return s;
 }
 template <typename R>
-__global__ void __cluster_dims__(kSumCtas, 1, 1) __launch_bounds__(1024) k_sum_reals(const R* __restrict__ x, int64_t n,
-                                                                                    double* __restrict__ out) {
-  __shared__ double sh[32], s_part[kSumCtas];
-  asm volatile("barrier.cluster.arrive.release;" ::: "memory");  // waited for below: every block runs
-  const int64_t i0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, step = (int64_t)kSumCtas * blockDim.x;
+__global__ void __launch_bounds__(kSumThreads) k_sum_reals(R* x, int64_t n, int64_t seg, double* __restrict__ out) {
+  __shared__ double sh[32];
+  x += blockIdx.x * seg;
+  n = min(seg, n - (int64_t)blockIdx.x * seg);
   double a = 0.0;
   bool add64 = true;
   if constexpr (sizeof(R) == 4) {
     float hi = 0.f, lo = 0.f, tail = 0.f;
 #pragma unroll 8
-    for (int64_t i = i0; i < n; i += step) {
+    for (int64_t i = threadIdx.x; i < n; i += kSumThreads) {
       float e, e2;
-      hi = two_sum(hi, __ldg(x + i), e);
+      hi = two_sum(hi, x[i], e);
       lo = two_sum(lo, e, e2);
       tail = __fadd_rn(tail, e2);
     }
@@ -284,28 +288,33 @@ __global__ void __cluster_dims__(kSumCtas, 1, 1) __launch_bounds__(1024) k_sum_r
     if (!add64) a = (double)hi + ((double)lo + (double)tail);
   }
   if (add64)
-    for (int64_t i = i0; i < n; i += step) a += (double)x[i];
-  a = block_sum(a, sh);
-  asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
-  if (threadIdx.x == 0) {
-    uint32_t dst;
-    asm volatile("mapa.shared::cluster.u32 %0, %1, 0;" : "=r"(dst) : "r"((uint32_t)__cvta_generic_to_shared(s_part + blockIdx.x)));
-    asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(dst), "d"(a) : "memory");
-  }
-  asm volatile("barrier.cluster.arrive.release;\n barrier.cluster.wait.acquire;" ::: "memory");
-  if (blockIdx.x == 0 && threadIdx.x == 0) {
-    double t = 0.0;
-    for (int c = 0; c < kSumCtas; ++c) t += s_part[c];
-    *out = t;
-  }
+    for (int64_t i = threadIdx.x; i < n; i += kSumThreads) a += (double)x[i];
+  a = block_sum(a, sh);  // its barriers: every thread has read its values
+  if (threadIdx.x == 0) *(gridDim.x == 1 ? out : reinterpret_cast<double*>(x)) = a;
+}
+// the sums of `blocks` <= kSumBlocks segments
+template <typename R>
+__global__ void __launch_bounds__(32) k_sum_segments(const R* x, int64_t seg, int blocks, double* __restrict__ out) {
+  double a = 0.0;
+  for (int b = threadIdx.x; b < blocks; b += 32) a += *reinterpret_cast<const double*>(x + b * seg);
+  for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
+  if (threadIdx.x == 0) *out = a;
 }
 
 template <typename R>
-cudaError_t launch_sum_reals(const R* x, int64_t n, double* out, cudaStream_t st) {
-  k_sum_reals<R><<<kSumCtas, 1024, 0, st>>>(x, n, out);
+cudaError_t launch_sum_reals(R* x, int64_t n, double* out, cudaStream_t st) {
+  // segments in whole kSumSegment, so that their sums are 8-byte aligned; the sum of
+  // a last segment of one float32 takes four bytes of the array's padding to 256
+  const int64_t seg = n <= kSumOne ? std::max<int64_t>(n, 1)
+                                   : kSumSegment * ((n + kSumSegment * kSumBlocks - 1) / (kSumSegment * kSumBlocks));
+  const int blocks = (int)std::max<int64_t>(1, (n + seg - 1) / seg);
+  k_sum_reals<R><<<blocks, kSumThreads, 0, st>>>(x, n, seg, out);
+  const cudaError_t e = cudaGetLastError();
+  if (e != cudaSuccess || blocks == 1) return e;
+  k_sum_segments<R><<<1, 32, 0, st>>>(x, seg, blocks, out);
   return cudaGetLastError();
 }
-template cudaError_t launch_sum_reals<float>(const float*, int64_t, double*, cudaStream_t);
-template cudaError_t launch_sum_reals<double>(const double*, int64_t, double*, cudaStream_t);
+template cudaError_t launch_sum_reals<float>(float*, int64_t, double*, cudaStream_t);
+template cudaError_t launch_sum_reals<double>(double*, int64_t, double*, cudaStream_t);
 
 }  // namespace sc

@@ -368,7 +368,7 @@ size_t lm_stats_doubles(int T, int64_t B);  // size of stat for any GPU of at mo
 size_t lm_part_doubles(int N);              // size of the per-tile partials
 cudaError_t launch_sum_cost(const double* cpart, int N, double* out, cudaStream_t st);
 template <typename R>
-cudaError_t launch_sum_reals(const R* x, int64_t n, double* out, cudaStream_t st);
+cudaError_t launch_sum_reals(R* x, int64_t n, double* out, cudaStream_t st);
 
 // residual_all.cu
 template <typename R>
