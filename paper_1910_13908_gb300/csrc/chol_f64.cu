@@ -9,7 +9,7 @@
 // steps of about 420 cycles (one reciprocal, one multiplier, one update
 // instruction), a triangular product and a symmetric one.
 //
-// A job's blocks: the first runs the diagonal chain (the walker), the
+// A job's blocks: one runs the diagonal chain (the walker), the
 // others take tasks as they open:
 //   P(i, j)     i >= j+2: L_ij = A_ij Linv_jj^T, then A_i,j+1 -= L_ij L_j+1,j^T
 //   B(I, K, j)  the 32x32 block of tile rows 2I, 2I+1 and tile columns 2K,
@@ -69,6 +69,7 @@ __device__ __forceinline__ bool csync_and(bool v) {
       : "memory");
   return r != 0;
 }
+constexpr int kTurnBlocks = 16;  // blocks per job up to which the walkers' places go round
 constexpr int kTLD = kNB64 + 2;  // row pitch of a tile in shared memory: consecutive rows start 4 banks apart
 
 // ---- the 136 entries of a lower triangle on 128 threads ----------------------------------
@@ -390,7 +391,7 @@ __device__ void walker64(double* A, size_t lda, int n, double* Linv, uint32_t* s
 }
 
 __global__ void __launch_bounds__(kBlock64) k_chol64(double* __restrict__ A0, int lda_, int n,
-                                                    double* __restrict__ Linv0, int per_job, size_t js, int* sync0,
+                                                    double* __restrict__ Linv0, int per_job, int sms, size_t js, int* sync0,
                                                     uint32_t* status0, LMState* lm0) {
   const int job = blockIdx.x / per_job;
   LMState* lm = job_ptr(lm0, js, job);
@@ -408,7 +409,13 @@ __global__ void __launch_bounds__(kBlock64) k_chol64(double* __restrict__ A0, in
   __shared__ int s_first;
   const int tid = threadIdx.x, warp = tid >> 5;
   if (tid == 0) {
-    s_first = atomicAdd(sv.fctr, 1) == 0;  // the first block to arrive
+    // The walker: the first block to arrive; of jobs with few blocks, which go
+    // round the SMs, another place in each round: with the first of every job
+    // and an even number of SMs, half of them or a quarter had the walkers and
+    // the others the work (304 jobs of 64 stations, two blocks each: 25.8 ms a
+    // factorisation, 20.0; 4 jobs, 152 blocks each, are faster the first way).
+    s_first = per_job > kTurnBlocks ? atomicAdd(sv.fctr, 1) == 0
+                                    : (int)blockIdx.x - job * per_job == job * per_job / sms % per_job;
     if (s_first) LeaveWalkerSm::publish(sv.sctr);
     W.failed = 0;
   }
@@ -714,10 +721,14 @@ cudaError_t launch_chol64(double* A, int lda, int nT, double* Linv, int* sync, u
   // up to four blocks per SM: the float64 pipes take about one, the others
   // cover claims, waits and loads (one block of four groups per SM with
   // blocks kept for P was 4% slower at order 1200 and 15% at 4096)
-  static const int resident = [] {
-    int dev = 0, sms = 0, per = 0;
+  static const int sms = [] {
+    int dev = 0, v = 0;
     cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev);
+    return std::max(1, v);
+  }();
+  static const int resident = [] {
+    int per = 0;
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_chol64, kBlock64, 0);
     return std::max(2, sms * std::min(std::max(per, 1), 4));
   }();
@@ -728,14 +739,19 @@ cudaError_t launch_chol64(double* A, int lda, int nT, double* Linv, int* sync, u
                               : cudaMemset2DAsync(sync, bt.js, 0, row, bt.G, st);
   if (e != cudaSuccess) return e;
   // per job: the walker and as many blocks as the first panel has tasks, at
-  // least one, within what is resident at once
+  // least one, within what is resident at once; of a large batch three, even if
+  // its last jobs then start when others are done: a job's walker keeps an SM
+  // little busy, and its one worker waits as much as it multiplies (64 stations,
+  // 304 jobs 18.2 ms with two workers, 14.6 with three; 400 jobs 26.7 with one,
+  // 17.5; 64x64 tiles in one list for all jobs, as before, took 14.3 and 18.8)
   const long long tasks = (long long)p_count64(n, 0) + b_count64(n, 0);
   const int total = max_ctas > 0 ? std::min(resident, max_ctas) : resident;
-  const int per_job = (int)std::max<long long>(2, std::min<long long>(1 + tasks, total / bt.G));
+  const int share = std::max(total / bt.G, max_ctas > 0 ? 2 : 4);
+  const int per_job = (int)std::max<long long>(2, std::min<long long>(1 + tasks, share));
   if ((long long)per_job * bt.G > (1LL << 30)) return cudaErrorInvalidValue;
   // not by launch_dep: blocks that come in while the assembly still runs crowd
   // on the SMs it has left, the walker among them (64 stations: 4.58 ms, 3.81)
-  k_chol64<<<per_job * bt.G, kBlock64, 0, st>>>(A, lda, n, Linv, per_job, bt.js, sync, status, lm);
+  k_chol64<<<per_job * bt.G, kBlock64, 0, st>>>(A, lda, n, Linv, per_job, sms, bt.js, sync, status, lm);
   return cudaGetLastError();
 }
 

@@ -6,7 +6,8 @@ on one cluster per job; a batch goes over to the general forms.  Jobs of 70
 stations have 15 tile pairs: 24 of them make 360, above the short form's line
 of two blocks per SM, and 24 clusters of 16 CTAs more than the GPU holds.  Of
 20 stations (3 pairs, 3 tile rows) 30 jobs stay below the first line and cross
-the second (30 clusters of 8 CTAs), and 110 cross both."""
+the second (30 clusters of 8 CTAs), and 110 cross both.  In float64 200 jobs have
+more blocks of the factorisation than the GPU holds."""
 import pytest
 
 torch = pytest.importorskip("torch")
@@ -32,7 +33,8 @@ def _job(N, T, F, K, seed, prec):
                   costs=torch.zeros(K, dtype=torch.float64, device="cuda"), ws=ws, stream=torch.cuda.current_stream())
 
 
-@pytest.mark.parametrize("n_jobs,N,prec", [(24, 70, "mixed"), (30, 20, "mixed"), (110, 20, "mixed"), (24, 70, "fp64")])
+@pytest.mark.parametrize("n_jobs,N,prec", [(24, 70, "mixed"), (30, 20, "mixed"), (110, 20, "mixed"), (24, 70, "fp64"),
+                                            (200, 20, "fp64")])
 def test_large_lockstep_batch_equals_jobs_alone(n_jobs, N, prec):
     prec = sc.SC_MIXED if prec == "mixed" else sc.SC_FP64
     shapes = [(N, 1 + i % 7, 1 + i % 3, 2, 100 + i) for i in range(n_jobs)]
